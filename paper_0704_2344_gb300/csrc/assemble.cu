@@ -147,12 +147,14 @@ __global__ void __launch_bounds__(256) k_assemble(const uint8_t* __restrict__ ma
                                                   const double2* __restrict__ tab, double2* __restrict__ val64,
                                                   float2* __restrict__ val32, float4* __restrict__ valdf,
                                                   double2* __restrict__ dinv64, float2* __restrict__ dinv32,
-                                                  float4* __restrict__ dinvdf, int n_act, int64_t stride,
+                                                  float4* __restrict__ dinvdf, int64_t stride,
                                                   unsigned abc, unsigned planes, int form_e,
+                                                  const int* __restrict__ rows, int n_rows,
                                                   int* __restrict__ status) {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int item = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
-    if (warp >= n_act) return;
+    if (item >= n_rows) return;
+    const int warp = rows ? rows[item] : item;  // the block row
     const int id = node_id[warp];
     const int i = id % (nx + 1), j = (id / (nx + 1)) % (ny + 1), k = id / ((nx + 1) * (ny + 1));
     // elements around the node (bit ex + 2ey + 4ez: element (i-1+ex, j-1+ey, k-1+ez))
@@ -325,7 +327,7 @@ __global__ void k_class_stencil(const double2* __restrict__ val64, int64_t strid
                                 const int* __restrict__ rep, StencilSet* __restrict__ S) {
     const int c = blockIdx.x, lane = threadIdx.x;
     const int r = rep[c];
-    const bool has = r != 0x7fffffff;
+    const bool has = r != 0x7f7f7f7f;
     double2 v[9];
     double amax = 0.0;
     if (has && lane < 27) {
@@ -418,6 +420,7 @@ static void system_free(fe_system* s) {
                       &s->dict_vals, &s->bicp_l,
                       &s->bicp_linv, &s->bicp_tpos, &s->bicp_tab, &s->bicp_lev, &s->bicp_nlev})
         dev_free(st, *b);
+    drop_patterns(s);
     s->bicp_n_sub = 0;
     s->n_dict = 0;
 }
@@ -502,81 +505,109 @@ fe_status fe_assemble(fe_ctx* ctx, const fe_mesh* m, double freq_hz, int32_t pre
             return fail(FE_ERR_CUDA);
         }
     }
+    // Rows of equal surroundings have equal blocks (patterns.cu): only the
+    // first row of each pattern is assembled and the others copy it.  Without
+    // patterns every row is assembled.
+    int* d_flags = (int*)ctx->small.ptr + 40;   // patterns, overflow, mismatch, least and largest cost, distinct blocks
+    int* d_totals = (int*)ctx->small.ptr + 48;  // sums over the rows: cost, explicit rows
+    DevBuf row_group;
+    auto fail_group = [&](fe_status e) {
+        dev_free(st, row_group);
+        return fail(e);
+    };
+    if ((e = group_rows(ctx, s, row_group, d_flags)) != FE_OK) return fail_group(e);
     const int threads = 256;
-    const unsigned blocks = (unsigned)(((int64_t)m->n_act * 32 + threads - 1) / threads);
+    const int n_asm = s->n_pat ? s->n_pat : m->n_act;
+    const unsigned blocks = (unsigned)(((int64_t)n_asm * 32 + threads - 1) / threads);
     k_assemble<<<blocks, threads, 0, st>>>((const uint8_t*)m->material.ptr, m->nx, m->ny, m->nz, m->n_mat,
                                            (const int*)m->node_id.ptr, (const int*)m->row_ptr.ptr,
                                            (const double2*)s->tables.ptr, (double2*)s->val64.ptr,
                                            (float2*)s->val32.ptr, (float4*)s->valdf.ptr, (double2*)s->dinv64.ptr,
-                                           (float2*)s->dinv32.ptr, (float4*)s->dinvdf.ptr, m->n_act, s->stride,
+                                           (float2*)s->dinv32.ptr, (float4*)s->dinvdf.ptr, s->stride,
                                            abc_faces(m->boundary), pack_planes(m->boundary),
-                                           s->formulation == FE_FORMULATION_E ? 1 : 0, d_status);
+                                           s->formulation == FE_FORMULATION_E ? 1 : 0,
+                                           s->n_pat ? (const int*)s->pat_first.ptr : nullptr, n_asm, d_status);
     {
         count_launches(1);
         cudaError_t ce = cudaGetLastError();
         if (ce != cudaSuccess) {
             set_error("k_assemble launch: %s", cudaGetErrorString(ce));
-            return fail(FE_ERR_CUDA);
+            return fail_group(FE_ERR_CUDA);
         }
     }
+    if (s->n_pat && (e = build_patterns(ctx, s, row_group, d_flags, d_totals)) != FE_OK) return fail_group(e);
+    dev_free(st, row_group);
     // regular-row classes and their stencils
     if ((e = dev_alloc(st, s->row_class, (size_t)m->n_act)) != FE_OK) return fail(e);
     if ((e = dev_alloc(st, s->stencil, sizeof(StencilSet))) != FE_OK) return fail(e);
     int* d_rep = (int*)ctx->small.ptr + 16;  // kMaxClasses ints
-    {
-        std::vector<int> big(kMaxClasses, 0x7fffffff);
-        cudaMemcpyAsync(d_rep, big.data(), kMaxClasses * sizeof(int), cudaMemcpyHostToDevice, st);
-        k_row_class<<<(unsigned)((m->n_act + 255) / 256), 256, 0, st>>>(
-            (const uint8_t*)m->material.ptr, m->nx, m->ny, m->nz, (const int*)m->node_id.ptr, m->n_act,
-            s->formulation == FE_FORMULATION_E ? 1 : 0, (signed char*)s->row_class.ptr, d_rep);
-        count_launches(1);
-        k_class_stencil<<<kMaxClasses, 32, 0, st>>>((const double2*)s->val64.ptr, s->stride,
-                                                    (const int*)m->row_ptr.ptr, d_rep, (StencilSet*)s->stencil.ptr);
-        count_launches(1);
-        // product cost prefixes, in units of one stored block of an explicit
-        // row: a general-stencil row costs 18 (complex64) or 27 (FP32 pairs,
-        // read through the block dictionary like an explicit row) such
-        // blocks, a diagonal-stencil row 10 or 9 (per-CTA product times
-        // measured on GB300 and fitted to these three row kinds)
-        // The third prefix counts the stored blocks of explicit rows only: a
-        // solve CTA packs its explicit rows' values at 9 times that prefix.
-        const int weights[3][3] = {{1, 18, 10}, {1, 27, 9}, {1, 0, 0}};
-        DevBuf* bufs[3] = {&s->cost_prefix, &s->cost_prefix_alu, &s->expl_prefix};
-        int* d_total = (int*)ctx->small.ptr + 24;
-        for (int k = 0; k < 3; ++k) {
-            if ((e = dev_alloc(st, *bufs[k], (size_t)(m->n_act + 1) * sizeof(int))) != FE_OK) return fail(e);
-            int* cp = (int*)bufs[k]->ptr;
-            k_row_cost<<<(unsigned)((m->n_act + 255) / 256), 256, 0, st>>>(
-                (const signed char*)s->row_class.ptr, (const StencilSet*)s->stencil.ptr, (const int*)m->row_ptr.ptr,
-                m->n_act, weights[k][0], weights[k][1], weights[k][2], cp);
-            count_launches(1);
-            if ((e = scan_exclusive(st, cp, cp, m->n_act, d_total + k, ctx->scan_tmp)) != FE_OK) return fail(e);
-            cudaMemcpyAsync(cp + m->n_act, d_total + k, sizeof(int), cudaMemcpyDeviceToDevice, st);
-        }
-        unsigned long long* d_counts = (unsigned long long*)((int*)ctx->small.ptr + 32);
-        cudaMemsetAsync(d_counts, 0, 3 * sizeof(unsigned long long), st);
-        k_class_counts<<<std::max(1, std::min(1024, (m->n_act + 255) / 256)), 256, 0, st>>>(
+    cudaMemsetAsync(d_rep, 0x7f, kMaxClasses * sizeof(int), st);
+    k_row_class<<<(unsigned)((m->n_act + 255) / 256), 256, 0, st>>>(
+        (const uint8_t*)m->material.ptr, m->nx, m->ny, m->nz, (const int*)m->node_id.ptr, m->n_act,
+        s->formulation == FE_FORMULATION_E ? 1 : 0, (signed char*)s->row_class.ptr, d_rep);
+    k_class_stencil<<<kMaxClasses, 32, 0, st>>>((const double2*)s->val64.ptr, s->stride, (const int*)m->row_ptr.ptr,
+                                                d_rep, (StencilSet*)s->stencil.ptr);
+    unsigned long long* d_counts = (unsigned long long*)((int*)ctx->small.ptr + 32);
+    cudaMemsetAsync(d_counts, 0, 3 * sizeof(unsigned long long), st);
+    k_class_counts<<<std::max(1, std::min(1024, (m->n_act + 255) / 256)), 256, 0, st>>>(
+        (const signed char*)s->row_class.ptr, (const StencilSet*)s->stencil.ptr, (const int*)m->row_ptr.ptr, m->n_act,
+        d_counts);
+    count_launches(3);
+    int* h = ctx->h_small;
+    if (s->n_pat && precision != FE_PREC_FP64 && (e = count_pattern_blocks(ctx, s, d_flags + 5)) != FE_OK)
+        return fail(e);
+    cudaMemcpyAsync(h + 32, d_counts, 20 * sizeof(int), cudaMemcpyDeviceToHost, st);
+    cudaError_t ce = cudaStreamSynchronize(st);
+    if (ce != cudaSuccess) {
+        set_error("row patterns: %s", cudaGetErrorString(ce));
+        return fail(FE_ERR_CUDA);
+    }
+    const unsigned long long* hc = (const unsigned long long*)(h + 32);
+    s->rows_general = (int64_t)hc[0];
+    s->rows_diagonal = (int64_t)hc[1];
+    s->blocks_explicit = (int64_t)hc[2];
+    if (s->n_pat) {
+        s->pat_cost_min = h[43];
+        s->pat_cost_max = h[44];
+        s->pat_cost_total = h[48];
+        s->n_expl = h[49];
+        s->n_dict = precision != FE_PREC_FP64 && !h[46] && h[45] <= kMaxDict ? h[45] : 0;
+        *out = s;
+        return FE_OK;
+    }
+    // Without patterns the products read the stored blocks, the class stencils
+    // and the block dictionary, and their rows are split by these costs, in
+    // units of one stored block of an explicit row: a general-stencil row
+    // costs 18 (complex64) or 27 (FP32 pairs, read through the block
+    // dictionary like an explicit row) such blocks, a diagonal-stencil row 10
+    // or 9 (per-CTA product times measured on GB300 and fitted to these three
+    // row kinds).  The third prefix counts the stored blocks of explicit rows
+    // only: a solve CTA packs its explicit rows' values at 9 times that prefix.
+    const int weights[3][3] = {{1, 18, 10}, {1, 27, 9}, {1, 0, 0}};
+    DevBuf* bufs[3] = {&s->cost_prefix, &s->cost_prefix_alu, &s->expl_prefix};
+    int* d_total = (int*)ctx->small.ptr + 24;
+    for (int k = 0; k < 3; ++k) {
+        if ((e = dev_alloc(st, *bufs[k], (size_t)(m->n_act + 1) * sizeof(int))) != FE_OK) return fail(e);
+        int* cp = (int*)bufs[k]->ptr;
+        k_row_cost<<<(unsigned)((m->n_act + 255) / 256), 256, 0, st>>>(
             (const signed char*)s->row_class.ptr, (const StencilSet*)s->stencil.ptr, (const int*)m->row_ptr.ptr,
-            m->n_act, d_counts);
+            m->n_act, weights[k][0], weights[k][1], weights[k][2], cp);
         count_launches(1);
-        cudaMemcpyAsync(ctx->h_small + 24, d_total, 2 * sizeof(int), cudaMemcpyDeviceToHost, st);
-        cudaMemcpyAsync(ctx->h_small + 32, d_counts, 3 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st);
-        cudaError_t ce = cudaStreamSynchronize(st);  // `big` must outlive the copy
-        if (ce != cudaSuccess) {
-            set_error("regular-row classes: %s", cudaGetErrorString(ce));
-            return fail(FE_ERR_CUDA);
-        }
-        s->cost_total = ctx->h_small[24];
-        s->cost_total_alu = ctx->h_small[25];
-        // bounds of one row's cost (an explicit row has 8 to 27 blocks)
-        for (int k = 0; k < 2; ++k) {
-            s->cost_min[k] = std::min({8 * weights[k][0], weights[k][1], weights[k][2]});
-            s->cost_max[k] = std::max({27 * weights[k][0], weights[k][1], weights[k][2]});
-        }
-        const unsigned long long* hc = (const unsigned long long*)(ctx->h_small + 32);
-        s->rows_general = (int64_t)hc[0];
-        s->rows_diagonal = (int64_t)hc[1];
-        s->blocks_explicit = (int64_t)hc[2];
+        if ((e = scan_exclusive(st, cp, cp, m->n_act, d_total + k, ctx->scan_tmp)) != FE_OK) return fail(e);
+        cudaMemcpyAsync(cp + m->n_act, d_total + k, sizeof(int), cudaMemcpyDeviceToDevice, st);
+    }
+    cudaMemcpyAsync(h + 24, d_total, 2 * sizeof(int), cudaMemcpyDeviceToHost, st);
+    ce = cudaStreamSynchronize(st);
+    if (ce != cudaSuccess) {
+        set_error("regular-row classes: %s", cudaGetErrorString(ce));
+        return fail(FE_ERR_CUDA);
+    }
+    s->cost_total = h[24];
+    s->cost_total_alu = h[25];
+    // bounds of one row's cost (an explicit row has 8 to 27 blocks)
+    for (int k = 0; k < 2; ++k) {
+        s->cost_min[k] = std::min({8 * weights[k][0], weights[k][1], weights[k][2]});
+        s->cost_max[k] = std::max({27 * weights[k][0], weights[k][1], weights[k][2]});
     }
     if ((e = build_block_dict(ctx, s)) != FE_OK) return fail(e);
     *out = s;
@@ -599,8 +630,9 @@ fe_status fe_system_info(const fe_system* s, fe_system_stats* out) {
     int64_t bytes = 0;
     for (const DevBuf* b : {&s->tables, &s->val64, &s->val32, &s->valdf, &s->dinv64, &s->dinv32, &s->dinvdf,
                             &s->row_class, &s->stencil, &s->cost_prefix, &s->cost_prefix_alu, &s->expl_prefix,
-                            &s->dict_idx, &s->dict_vals, &s->bicp_l,
-                            &s->bicp_linv, &s->bicp_tpos, &s->bicp_tab, &s->bicp_lev, &s->bicp_nlev})
+                            &s->dict_idx, &s->dict_vals, &s->pat_first, &s->pat_id, &s->pat_tab, &s->pat_t64,
+                            &s->pat_t32, &s->pat_tdf, &s->pat_cost, &s->pat_list, &s->bicp_l, &s->bicp_linv,
+                             &s->bicp_tpos, &s->bicp_tab, &s->bicp_lev, &s->bicp_nlev})
         bytes += (int64_t)b->bytes;
     out->device_bytes = bytes + half_bytes(s);
     return FE_OK;

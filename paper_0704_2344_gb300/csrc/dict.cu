@@ -29,13 +29,6 @@ constexpr int kDictTableBits = 17;
 constexpr int kDictTable = 1 << kDictTableBits;
 constexpr int kDictProbes = 64;
 
-__device__ __forceinline__ unsigned long long mix64(unsigned long long z) {
-    // the finaliser of the SplitMix64 generator (Steele, Lea and Flood, 2014)
-    z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ull;
-    z = (z ^ (z >> 27)) * 0x94d049bb133111ebull;
-    return z ^ (z >> 31);
-}
-
 __device__ __forceinline__ unsigned long long block_hash(const double2* __restrict__ val, int64_t stride, int64_t s) {
     unsigned long long h = 0x9e3779b97f4a7c15ull;
 #pragma unroll
@@ -99,6 +92,46 @@ __global__ void k_dict_fill(const int* __restrict__ rep_of_id, int n_dict, int64
     const int64_t src = q * stride + rep_of_id[d];
     if (d32) d32[i] = val32[src];
     if (ddf) ddf[i] = valdf[src];
+}
+
+// Counts the distinct blocks of a system with row patterns: every block
+// occurs in the first row of some pattern, so only those rows are inserted
+// (one warp per pattern).
+__global__ void k_dict_count(const double2* __restrict__ val, int64_t stride, const int* __restrict__ first_of_id,
+                             int n_pat, const int* __restrict__ row_ptr, unsigned long long* __restrict__ keys,
+                             int* __restrict__ d_flags) {
+    const int p = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    if (p >= n_pat) return;
+    const int s0 = row_ptr[first_of_id[p]], s1 = row_ptr[first_of_id[p] + 1];
+    if (s0 + lane >= s1) return;
+    const unsigned long long h = block_hash(val, stride, s0 + lane);
+    unsigned t = (unsigned)(h >> (64 - kDictTableBits));
+    for (int probe = 0; probe < kDictProbes; ++probe, t = (t + 1) & (kDictTable - 1)) {
+        const unsigned long long prev = atomicCAS(keys + t, 0ull, h);
+        if (prev == 0ull) atomicAdd(d_flags, 1);
+        if (prev == 0ull || prev == h) return;
+    }
+    atomicExch(d_flags + 1, 1);
+}
+
+// d_flags: the count and an overflow mark, on the device.
+fe_status count_pattern_blocks(fe_ctx* ctx, const fe_system* s, int* d_flags) {
+    cudaStream_t st = ctx->stream;
+    DevBuf keys;
+    FE_TRY(dev_alloc(st, keys, (size_t)kDictTable * sizeof(unsigned long long)));
+    cudaMemsetAsync(keys.ptr, 0, (size_t)kDictTable * sizeof(unsigned long long), st);
+    cudaMemsetAsync(d_flags, 0, 2 * sizeof(int), st);
+    k_dict_count<<<(unsigned)((s->n_pat * 32 + 255) / 256), 256, 0, st>>>(
+        (const double2*)s->val64.ptr, s->stride, (const int*)s->pat_first.ptr, s->n_pat,
+        (const int*)s->mesh->row_ptr.ptr, (unsigned long long*)keys.ptr, d_flags);
+    count_launches(1);
+    dev_free(st, keys);
+    const cudaError_t ce = cudaGetLastError();
+    if (ce != cudaSuccess) {
+        set_error("distinct blocks: %s", cudaGetErrorString(ce));
+        return FE_ERR_CUDA;
+    }
+    return FE_OK;
 }
 
 fe_status build_block_dict(fe_ctx* ctx, fe_system* s) {

@@ -186,6 +186,18 @@ struct fe_system {
     int n_dict = 0;
     int cost_min[2] = {1, 1}, cost_max[2] = {1, 1};  // bounds of one row's cost (complex64, FP32 pairs)
     int64_t rows_general = 0, rows_diagonal = 0, blocks_explicit = 0;  // rows per product path
+    // Row patterns (patterns.cuh): the distinct block rows as term lists, and
+    // each row's pattern.  n_pat = 0: none (the products read stored blocks).
+    int n_pat = 0;
+    int pat_cost_min = 1, pat_cost_max = 1;  // bounds of one row's cost
+    int n_expl = 0;                  // explicit rows: rows whose pattern is not of real diagonal blocks
+    int64_t pat_cost_total = 0;
+    fe::DevBuf pat_first;                // int [n_pat]: first row of each pattern
+    fe::DevBuf pat_id;               // uint16 [n_act]
+    fe::DevBuf pat_tab;              // int4 [n_pat]: (first term triple, n_re, n_im, real diagonal blocks)
+    fe::DevBuf pat_t64, pat_t32, pat_tdf;  // terms [n_pat * kPatStride * 3]: double2 / float2 / float4
+    fe::DevBuf pat_cost;             // int [n_act + 1]: prefix sum of the rows' product cost
+    fe::DevBuf pat_list;             // int [n_expl]: the explicit rows, ascending
     // Block incomplete Cholesky factor (Section 3.1.5.3): node rows split into
     // bicp_n_sub contiguous bands, floor(b n / S) <= I < floor((b + 1) n / S),
     // one per CTA of the solve; L L^T reproduces A on the lower node-block
@@ -202,9 +214,20 @@ struct fe_system {
 };
 
 namespace fe {
+// the finaliser of the SplitMix64 generator (Steele, Lea and Flood, 2014)
+__device__ __forceinline__ unsigned long long mix64(unsigned long long z) {
+    z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ull;
+    z = (z ^ (z >> 27)) * 0x94d049bb133111ebull;
+    return z ^ (z >> 31);
+}
 constexpr int kMaxClasses = 4;
 constexpr int kMaxDict = 4096;  // distinct blocks a dictionary may hold
 fe_status build_block_dict(fe_ctx* ctx, fe_system* s);
+fe_status count_pattern_blocks(fe_ctx* ctx, const fe_system* s, int* d_flags);
+fe_status group_rows(fe_ctx* ctx, fe_system* s, DevBuf& row_group, int* d_flags);
+fe_status build_patterns(fe_ctx* ctx, fe_system* s, const DevBuf& row_group, int* d_flags, int* d_totals);
+void drop_patterns(fe_system* s);
+
 // Per-class stencils of regular rows, indexed [class][alpha][block k][beta];
 // kind: 0 = no regular row, 1 = general complex blocks, 2 = real diagonal
 // blocks (the homogeneous interior with eps_r = 1 and s = 1); dval holds the

@@ -28,7 +28,7 @@
 #include <thread>
 #include <unordered_map>
 
-#include "fe_internal.cuh"
+#include "patterns.cuh"
 
 namespace fe {
 struct SolveJob;
@@ -111,11 +111,13 @@ int64_t estimate_bytes(const fe_mesh_desc& d, int nrhs, int width, int prec, int
     // complex128 values, plus the complex64 or FP32-pair copy
     const int64_t per_entry = prec == FE_PREC_FP64 ? 16 : (prec == FE_PREC_MIXED ? 24 : 32);
     const int64_t sys = 9 * stride * per_entry + 9 * nodes * 24 + nodes * 13 + 65536;
+    // row patterns: term lists, the row tables and what their construction holds
+    const int64_t pat = (int64_t)pat_limit(nodes) * kPatStride * 3 * per_entry + 64 * nodes + (1 << 18);
     const int64_t rhs = 3 * nodes * (int64_t)nrhs * 16;
     // the packed explicit rows of a single-column launch: at most every block
     const int64_t pk = (width == 1 && prec != FE_PREC_FP64) ? 9 * nnzb : 0;
     const int64_t ws = (int64_t)workspace_bytes(3 * nodes, width, prec, 2 * num_sms, pk);
-    return (mesh + sys + rhs + ws) * 11 / 10 + (1 << 20);
+    return (mesh + sys + pat + rhs + ws) * 11 / 10 + (1 << 20);
 }
 
 }  // namespace

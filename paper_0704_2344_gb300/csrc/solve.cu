@@ -23,7 +23,7 @@
 #include <mutex>
 #include <new>
 #include <tuple>
-#include "solve_kernels.cuh"
+#include "solve_pattern.cuh"
 
 namespace fe {
 
@@ -34,6 +34,19 @@ extern template fe_status dispatch<DFloat>(fe_ctx*, int, SolveParams&);
 extern template fe_status launch_jobs_w<double>(fe_ctx*, int, SolveJob* const*, const int*, int, cudaStream_t, const int*);
 extern template fe_status launch_jobs_w<float>(fe_ctx*, int, SolveJob* const*, const int*, int, cudaStream_t, const int*);
 extern template fe_status launch_jobs_w<DFloat>(fe_ctx*, int, SolveJob* const*, const int*, int, cudaStream_t, const int*);
+
+// and, for systems with row patterns, in solve_pat_fp64.cu and its siblings
+extern template fe_status dispatch_pat<double>(fe_ctx*, int, SolveParams&);
+extern template fe_status dispatch_pat<float>(fe_ctx*, int, SolveParams&);
+extern template fe_status dispatch_pat<DFloat>(fe_ctx*, int, SolveParams&);
+extern template fe_status launch_pat_jobs<double>(fe_ctx*, int, SolveJob* const*, const int*, int, cudaStream_t, const int*);
+extern template fe_status launch_pat_jobs<float>(fe_ctx*, int, SolveJob* const*, const int*, int, cudaStream_t, const int*);
+extern template fe_status launch_pat_jobs<DFloat>(fe_ctx*, int, SolveJob* const*, const int*, int, cudaStream_t, const int*);
+
+template <typename T>
+static fe_status run_solve(fe_ctx* ctx, int R, SolveParams& P) {
+    return P.pat_id ? dispatch_pat<T>(ctx, R, P) : dispatch<T>(ctx, R, P);
+}
 
 // Column gather / scatter between [n_dof][nrhs] and a [n_dof][R] tile.
 __global__ void k_gather_cols(const double2* __restrict__ src, int lds, int c0, int ncols, double2* __restrict__ dst,
@@ -66,7 +79,7 @@ static int pick_tile(int nrhs, int requested) {
 
 static void free_workspace(cudaStream_t st, Workspace& w) {
     for (DevBuf* b : {&w.b, &w.x, &w.r, &w.u, &w.p, &w.s, &w.uM, &w.pM, &w.w, &w.partial, &w.result, &w.sync, &w.rep,
-                      &w.trace, &w.pk, &w.state})
+                      &w.trace, &w.pk, &w.state, &w.pat})
         dev_free(st, *b);
 }
 
@@ -119,13 +132,19 @@ static fe_status with_inner_type(int prec, F&& f) {
 // most kDictSmemMax bytes (it is copied into every CTA's shared memory).
 constexpr size_t kDictSmemMax = 64 * 1024;
 static bool dict_usable(const fe_system* s, int prec, int R) {
-    return R == 1 && prec != FE_PREC_FP64 && s->n_dict > 0 &&
+    return R == 1 && prec != FE_PREC_FP64 && s->dict_vals.ptr && s->n_dict > 0 &&
            (size_t)s->n_dict * 9 * inner_bytes(prec) <= kDictSmemMax;
 }
 
 static int64_t packed_entries(const fe_system* s, int prec, int R) {
-    if (R != 1 || prec == FE_PREC_FP64 || !s->expl_prefix.ptr || dict_usable(s, prec, R)) return 0;
+    if (R != 1 || prec == FE_PREC_FP64 || s->n_pat || !s->expl_prefix.ptr || dict_usable(s, prec, R)) return 0;
     return 9 * s->blocks_explicit;
+}
+
+// Reduction partials of a launch on the row patterns (solve_pattern.cuh),
+// which runs at most one CTA per SM, half of max_cta.
+static size_t pat_partial_bytes(int max_cta, int R) {
+    return (size_t)((max_cta + 1) / 2) * kPatNV * R * 2 * sizeof(double);
 }
 
 static fe_status alloc_workspace(cudaStream_t st, int64_t n_dof, int R, int prec, int max_cta, Workspace& w,
@@ -139,7 +158,7 @@ static fe_status alloc_workspace(cudaStream_t st, int64_t n_dof, int R, int prec
                     std::make_pair(&w.pM, split_copies(prec, R) ? nv * esz : (size_t)16), std::make_pair(&w.w, nv * esz),
                     std::make_pair(&w.partial, (size_t)max_cta * kMaxNV * R * sizeof(double)),
                     std::make_pair(&w.result, (size_t)kMaxNV * R * sizeof(double)),
-                    std::make_pair(&w.sync, sync_bytes(max_cta)),
+                    std::make_pair(&w.pat, pat_partial_bytes(max_cta, R)), std::make_pair(&w.sync, sync_bytes(max_cta)),
                     std::make_pair(&w.rep, (size_t)R * (3 * sizeof(int) + sizeof(double)) + 64)}) {
         const fe_status e = dev_alloc(st, *pr.first, pr.second);
         if (e != FE_OK) {
@@ -162,7 +181,8 @@ size_t workspace_bytes(int64_t n_dof, int R, int prec, int max_cta, int64_t pk_e
     const size_t nv = (size_t)n_dof * R;
     const size_t esz = inner_bytes(prec);
     return nv * (6 * sizeof(double2) + (split_copies(prec, R) ? 3 : 1) * esz) + (size_t)(max_cta + 1) * kMaxNV * R * sizeof(double) +
-           (size_t)R * 32 + 4096 + (size_t)pk_entries * esz;
+           (size_t)R * 32 + 4096 + (size_t)pk_entries * esz +
+           pat_partial_bytes(max_cta, R);
 }
 
 // Solve parameters for a tile of R columns held in workspace w (n_cta and the
@@ -191,6 +211,23 @@ static void fill_params(SolveParams& P, const fe_system* s, const Workspace& w, 
     P.cost_total = classes ? (df ? s->cost_total_alu : s->cost_total) : (int64_t)m->n_act;
     P.cost_min = classes ? s->cost_min[df ? 1 : 0] : 1;
     P.cost_max = classes ? s->cost_max[df ? 1 : 0] : 1;
+    if (s->n_pat && !(o.preconditioner == FE_PRECOND_BICP && fp64)) {
+        P.pat_id = (const uint16_t*)s->pat_id.ptr;
+        P.pat_tab = (const int4*)s->pat_tab.ptr;
+        P.pat_first = (const int*)s->pat_first.ptr;
+        P.pat_partial = (double*)w.pat.ptr;
+        P.pat_terms = fp64 ? s->pat_t64.ptr : (df ? s->pat_tdf.ptr : s->pat_t32.ptr);
+        P.pat_terms64 = (const double2*)s->pat_t64.ptr;
+        P.node_id = (const int*)m->node_id.ptr;
+        P.node_rank = (const int*)m->node_rank.ptr;
+        P.pat_sy = m->nx + 1;
+        P.pat_sz = (m->nx + 1) * (m->ny + 1);
+        P.pat_nz1 = m->nz + 1;
+        P.cost_prefix = (const int*)s->pat_cost.ptr;
+        P.cost_total = s->pat_cost_total;
+        P.cost_min = s->pat_cost_min;
+        P.cost_max = s->pat_cost_max;
+    }
     P.b = (const double2*)w.b.ptr;
     P.x = (double2*)w.x.ptr;
     P.r = (double2*)w.r.ptr;
@@ -255,10 +292,11 @@ static fe_status solve_tiles(fe_ctx* ctx, const fe_system* s, int nrhs, int ldb,
 // ---------------------------------------------------------------------------
 // Autotuner of the tile width and the grid of multi-column solves.  A trial
 // is a real solve of the first columns capped at kTuneIters iterations; its
-// measure is device time per column and iteration.  Choices are cached per
+// measure is the device time of one iteration of all columns.  Choices are cached per
 // system shape for the life of the process.
 // ---------------------------------------------------------------------------
 constexpr int kTuneIters = 32;
+constexpr double kTuneTie = 0.05;
 
 struct TuneKey {
     int64_t n_dof, nnzb;
@@ -292,11 +330,12 @@ static fe_status autotune(fe_ctx* ctx, const fe_system* s, int nrhs, const doubl
     fe_solve_opts t = o;
     t.max_iter = kTuneIters;
     t.tol = 1e-300;  // trials never converge early
-    double best = 1e300;
-    int bestR = top, bestC = ctx->num_sms;
+    double best = 1e300, per[3] = {1e300, 1e300, 1e300};
+    int bestR = top, bestC = ctx->num_sms, cta[3] = {ctx->num_sms, ctx->num_sms, ctx->num_sms};
     fe_status e = FE_OK;
+    const int cols = std::min(nrhs, 32);
     const int grids[2] = {ctx->num_sms, std::max(1, ctx->num_sms * 3 / 4)};
-    for (int W = 8; W <= top && e == FE_OK; W *= 2)
+    for (int k = 0, W = 8; W <= top && e == FE_OK; ++k, W *= 2)
         for (int g = 0; g < 2 && e == FE_OK; ++g) {
             const fe_status es = solve_tiles(ctx, s, std::min(nrhs, W), nrhs, d_b, (double2*)xt.ptr, false, t, nullptr,
                                              W, grids[g]);
@@ -306,13 +345,23 @@ static fe_status autotune(fe_ctx* ctx, const fe_system* s, int nrhs, const doubl
             }
             const fe_solve_stats& st = ctx->last_solve;
             *tune_ms += st.kernel_ms;
-            // real columns only: the zero columns of a padded tile are done at once
-            const double per = st.inner_iters > 0 ? st.kernel_ms / (double)st.inner_iters : 1e300;
-            if (per < best) {
-                best = per;
-                bestR = W;
-                bestC = grids[g];
+            // device time of one iteration of all columns: a last tile that is
+            // partly padding costs a launch like the others
+            const double its = (double)st.inner_iters / std::min(nrhs, W);
+            const double all = its > 0 ? st.kernel_ms / its * ((cols + W - 1) / W) : 1e300;
+            if (all < per[k]) {
+                per[k] = all;
+                cta[k] = grids[g];
             }
+            best = std::min(best, all);
+        }
+    // the widest tile within kTuneTie of the fastest: it also saves launches,
+    // column copies, true-residual passes and host round trips, which the
+    // trials do not show
+    for (int k = 0, W = 8; W <= top; ++k, W *= 2)
+        if (per[k] < 1e300 && per[k] <= best * (1.0 + kTuneTie)) {
+            bestR = W;
+            bestC = cta[k];
         }
     dev_free(ctx->stream, xt);
     if (e != FE_OK) return e;
@@ -377,7 +426,7 @@ static fe_status solve_tiles(fe_ctx* ctx, const fe_system* s, int nrhs, int ldb,
         fill_params(P, s, w, R, prec, o, use_x0);
         P.n_cta_req = n_cta_req;
         int* ri = P.rep_status;
-        e = with_inner_type(prec, [&](auto* tag) { return dispatch<std::remove_pointer_t<decltype(tag)>>(ctx, R, P); });
+        e = with_inner_type(prec, [&](auto* tag) { return run_solve<std::remove_pointer_t<decltype(tag)>>(ctx, R, P); });
         if (e != FE_OK) break;
         const unsigned gs = (unsigned)((n_dof * nc + 255) / 256);
         k_scatter_cols<<<gs, 256, 0, st>>>((const double2*)w.x.ptr, R, nc, d_x, ldb, c0, n_dof);
@@ -537,9 +586,25 @@ fe_status jobs_launch(fe_ctx* ctx, SolveJob* const* jobs, const int* n_cta, int 
         set_error("jobs: %lld CTAs exceed one per SM", (long long)total);
         return FE_ERR_INVALID_ARG;
     }
-    return with_inner_type(prec, [&](auto* tag) {
-        return launch_jobs_w<std::remove_pointer_t<decltype(tag)>>(ctx, R, jobs, n_cta, n, stream, seg_iters);
-    });
+    // systems with and without row patterns run different kernels, one after
+    // the other on the stream
+    for (int pat = 1; pat >= 0; --pat) {
+        std::vector<SolveJob*> js;
+        std::vector<int> ctas, segs;
+        for (int i = 0; i < n; ++i)
+            if ((jobs[i]->P.pat_id != nullptr) == (pat == 1)) {
+                js.push_back(jobs[i]);
+                ctas.push_back(n_cta[i]);
+                segs.push_back(seg_iters ? seg_iters[i] : 0);
+            }
+        if (js.empty()) continue;
+        FE_TRY(with_inner_type(prec, [&](auto* tag) {
+            using T = std::remove_pointer_t<decltype(tag)>;
+            return pat ? launch_pat_jobs<T>(ctx, R, js.data(), ctas.data(), (int)js.size(), stream, segs.data())
+                       : launch_jobs_w<T>(ctx, R, js.data(), ctas.data(), (int)js.size(), stream, segs.data());
+        }));
+    }
+    return FE_OK;
 }
 
 // A job's progress after a launch, from its state block: whether the solve
@@ -604,8 +669,9 @@ fe_status job_collect(fe_ctx* ctx, SolveJob* j, fe_complex* x_host, fe_solve_rep
 // device address (it is a host-side stand-in); the address is looked up once
 // per device with cudaGetSymbolAddress while that device is current.
 // ---------------------------------------------------------------------------
-constexpr size_t kStaticScratchBytes = (size_t)32 << 20;  // 32 MiB per device
-static __device__ __align__(256) unsigned char g_solve_scratch[kStaticScratchBytes];
+constexpr size_t kStaticScratchBytes = (size_t)32 << 20;  // 32 MiB per device for what the documented need counts
+constexpr size_t kStaticReduceBytes = (size_t)2 << 20;    // and a launch's reduction partials (up to 32 columns)
+static __device__ __align__(256) unsigned char g_solve_scratch[kStaticScratchBytes + kStaticReduceBytes];
 constexpr int kMaxDevices = 64;
 static void* g_scratch_addr[kMaxDevices] = {nullptr};
 
@@ -845,6 +911,12 @@ fe_status fe_solve_rhs_noalloc(fe_ctx* ctx, const fe_system* s, int32_t nrhs, co
                   off, kStaticScratchBytes);
         return FE_ERR_INVALID_ARG;
     }
+    off = kStaticScratchBytes;
+    take(w.pat, pat_partial_bytes(max_cta, R));
+    if (off > kStaticScratchBytes + kStaticReduceBytes) {
+        set_error("fe_solve_rhs_noalloc: the reduction partials do not fit the static array");
+        return FE_ERR_INVALID_ARG;
+    }
     cudaStream_t st = ctx->stream;
     {
         const cudaError_t ce = cudaMemsetAsync(w.sync.ptr, 0, sync_bytes(ctx->num_sms), st);  // the array keeps old contents
@@ -861,7 +933,7 @@ fe_status fe_solve_rhs_noalloc(fe_ctx* ctx, const fe_system* s, int32_t nrhs, co
     int* ri = P.rep_status;
     double* rrel = P.rep_rel;
     ctx->last_solve = fe_solve_stats{};
-    FE_TRY(with_inner_type(prec, [&](auto* tag) { return dispatch<std::remove_pointer_t<decltype(tag)>>(ctx, R, P); }));
+    FE_TRY(with_inner_type(prec, [&](auto* tag) { return run_solve<std::remove_pointer_t<decltype(tag)>>(ctx, R, P); }));
     SyncState hs{};
     int h_ri[3 * 32];
     double h_rel[32];

@@ -1,10 +1,13 @@
 // Device code of the persistent solve and its launch templates, shared by
 // the host logic (solve.cu) and by one translation unit per product
 // arithmetic (solve_fp64.cu, solve_mixed.cu, solve_df.cu) that instantiates
-// the kernels, so that the three compile in parallel.
+// the kernels, so that the three compile in parallel.  Systems with row
+// patterns and block Jacobi, the common case, run solve_pattern.cuh instead;
+// this file serves the others (too many distinct rows, or the block
+// incomplete Cholesky preconditioner).
 #pragma once
 
-#include "krylov.cuh"
+#include "patterns.cuh"
 
 #include <algorithm>
 #include <cstdlib>
@@ -45,7 +48,7 @@ struct ColState {
     float4 a4, na4, b4;
     float4 gam4, igam4, ial4;  // FP32-pair solves: gamma, 1/gamma, 1/alpha as pairs
     long long xd[4];           // expanded recurrence: u^T s and p^T s of the last update (the raw 8-byte slots)
-    int active, done, status, iters, outer, first, refresh, repl, pass_it, pad2[3];
+    int active, done, status, iters, outer, first, refresh, repl, pass_it, kept, pad2[2];
 };
 struct JobState {
     int started;   // a segment has run (the next one resumes)
@@ -129,6 +132,20 @@ struct SolveParams {
     const uint16_t* dict_idx;  // [nnzb] dictionary index of each stored block
     const void* dictM;         // [n_dict * 9] distinct blocks in the inner precision
     int n_dict;
+    // Row patterns (solve_pattern.cuh); NULL: this file's kernels run the solve.
+    const uint16_t* pat_id;
+    const int4* pat_tab;
+    const int* pat_first;
+    const void* pat_terms;       // terms in the inner precision
+    const double2* pat_terms64;  // FP64 terms (true residual)
+    const int* node_id;
+    const int* node_rank;
+    int pat_sy, pat_sz, pat_nz1;  // nodes per grid line and plane, planes
+    int pat_rows_max;             // rows a CTA's shared row tables hold (0: no row tables)
+    int pat_terms_max;            // terms its shared copy holds
+    int pat_vec_max;              // work items whose vectors it keeps in shared memory (0: none)
+    double* pat_partial;          // partials of the reductions, two buffers
+    int64_t pat_half;             // values per buffer
     int* rep_status;
     int* rep_iters;
     int* rep_outer;
@@ -1898,7 +1915,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 }
 
 struct Workspace {
-    DevBuf b, x, r, u, p, s, uM, pM, w, partial, result, sync, rep, trace, pk, state;
+    DevBuf b, x, r, u, p, s, uM, pM, w, partial, result, sync, rep, trace, pk, state, pat;
 };
 
 constexpr size_t kSmemBudget = 200 * 1024;  // dynamic; static shared memory adds ~20 KB

@@ -1,6 +1,6 @@
 // Standalone sparse products y = A x (fe_spmv): the Krylov loop's product
 // (Section 3.1.5.1) as its own entry point, for one or several vectors.
-#include "krylov.cuh"
+#include "patterns.cuh"
 
 #include <algorithm>
 #include <cstdint>
@@ -349,6 +349,123 @@ static void launch_spmv_warp(int R, unsigned blocks, cudaStream_t st, const C* v
     }
 }
 
+// y = A x from the row patterns, R columns (R = 0: nrhs of them).  The matrix
+// is a few hundred kilobytes of terms that stay in L1 and L2, so the product
+// moves the vectors and the row tables only: the 80^3 aircraft's complex64
+// product reads 25 MB of vectors instead of 1.1 GB of blocks.
+// One thread per (row, component, column), so that the lanes of a warp read
+// consecutive vector entries; the first blocks take the explicit rows
+// (collected in a list, so that a warp holds rows of like length), the others
+// sweep all rows for the real diagonal ones.  kTile (complex64, R >= 8): the
+// sweep takes four consecutive rows per thread, which share two of every
+// three vector entries along a grid line; the product is then bound by the L1
+// traffic of those entries.
+template <typename C, int R_, bool kTile>
+__global__ void __launch_bounds__(256) k_spmv_pat(PatView<C> V, int n_rows, const int* __restrict__ list, int n_expl,
+                                                  int expl_blocks, int nrhs, const C* __restrict__ x,
+                                                  C* __restrict__ y) {
+    const int R = R_ ? R_ : nrhs;
+    auto load = [&](size_t i) { return __ldg(x + i); };
+    if ((int)blockIdx.x < expl_blocks) {
+        const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+        const int64_t d = e / R;
+        const int c = (int)(e - d * R), i = (int)(d / 3), al = (int)(d - 3 * (int64_t)i);
+        if (i >= n_expl) return;
+        const int row = __ldg(list + i);
+        const int4 t = __ldg(V.tab + __ldg(V.id + row));
+        const LineRanks base{V.node_rank + __ldg(V.node_id + row), V.sy, V.sz};
+        TermAcc<C> acc;
+        pattern_terms<C>(acc, V.terms + (size_t)t.x * 3 + al, t.y, t.z, R, c, base, load);
+        y[((size_t)3 * row + al) * R + c] = acc.result_norm();
+        return;
+    }
+    const int64_t e = (int64_t)(blockIdx.x - expl_blocks) * blockDim.x + threadIdx.x;
+    const int64_t d = e / R;
+    const int c = (int)(e - d * R);
+    auto one_row = [&](int row, int al) {
+        const int4 t = __ldg(V.tab + __ldg(V.id + row));
+        if (!t.w) return;
+        const LineRanks base{V.node_rank + __ldg(V.node_id + row), V.sy, V.sz};
+        TermAcc<C> acc;
+        pattern_diag<C, true>(acc, V.terms + (size_t)t.x * 3 + al, al, R, c, base, load);
+        y[((size_t)3 * row + al) * R + c] = acc.result_norm();
+    };
+    if constexpr (!kTile) {
+        const int row = (int)(d / 3);
+        if (row < n_rows) one_row(row, (int)(d - 3 * (int64_t)row));
+    } else {
+        const int r0 = 4 * (int)(d / 3), al = (int)(d % 3);
+        if (r0 >= n_rows) return;
+        const int id0 = __ldg(V.id + r0);
+        bool tile = r0 + 3 < n_rows;
+        if (tile)
+            tile = __ldg(V.id + r0 + 1) == id0 && __ldg(V.id + r0 + 2) == id0 && __ldg(V.id + r0 + 3) == id0 &&
+                   __ldg(V.node_id + r0 + 3) - __ldg(V.node_id + r0) == 3;
+        const int4 t = __ldg(V.tab + id0);
+        if (tile && !t.w) return;
+        if (!tile) {
+            for (int row = r0; row < min(r0 + 4, n_rows); ++row) one_row(row, al);
+            return;
+        }
+        const C* terms = V.terms + (size_t)t.x * 3 + al;
+        const LineRanks base{V.node_rank + __ldg(V.node_id + r0), V.sy, V.sz};
+        TermAcc<C> acc[4];
+        C own[4];
+        auto line = [&](int m, bool centre) {
+            const C* xp = x + ((size_t)(base(m) + al) * R + c) - 3 * R;
+            C v[6];
+#pragma unroll
+            for (int k = 0; k < 6; ++k) v[k] = __ldg(xp + 3 * k * R);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                if (centre && k == 1) continue;
+                const C w = __ldg(terms + 9 * m + 3 * k);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[j].add_re(w, v[j + k]);
+            }
+            if (centre)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) own[j] = v[j + 1];
+        };
+#pragma unroll 2
+        for (int k = 0; k < 8; ++k) line(k + (k >= 4), false);
+        line(4, true);  // the rows' own entries last
+        const C w = __ldg(terms + 39);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[j].add_re(w, own[j]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) y[((size_t)3 * (r0 + j) + al) * R + c] = acc[j].result_norm();
+    }
+}
+
+template <typename C, int R, bool kTile>
+static void launch_spmv_pat_t(cudaStream_t st, const PatView<C>& V, const fe_system* s, int nrhs, const C* x, C* y) {
+    const int n = s->mesh->n_act;
+    const int64_t expl = ((int64_t)s->n_expl * 3 * nrhs + 255) / 256;
+    const int64_t rows = kTile ? ((int64_t)n + 3) / 4 : n;
+    const int64_t all = (rows * 3 * nrhs + 255) / 256;
+    k_spmv_pat<C, R, kTile><<<(unsigned)(expl + all), 256, 0, st>>>(V, n, (const int*)s->pat_list.ptr, s->n_expl,
+                                                                   (int)expl, nrhs, x, y);
+}
+
+template <typename C>
+static void launch_spmv_pat(cudaStream_t st, const fe_system* s, const void* terms, int nrhs, const C* x, C* y) {
+    const fe_mesh* m = s->mesh;
+    const PatView<C> V{(const uint16_t*)s->pat_id.ptr, (const int4*)s->pat_tab.ptr, (const C*)terms,
+                       (const int*)m->node_id.ptr,     (const int*)m->node_rank.ptr, m->nx + 1,
+                       (m->nx + 1) * (m->ny + 1)};
+    constexpr bool kT = std::is_same<C, float2>::value;
+    switch (nrhs) {
+        case 1: launch_spmv_pat_t<C, 1, false>(st, V, s, nrhs, x, y); break;
+        case 2: launch_spmv_pat_t<C, 2, false>(st, V, s, nrhs, x, y); break;
+        case 4: launch_spmv_pat_t<C, 4, false>(st, V, s, nrhs, x, y); break;
+        case 8: launch_spmv_pat_t<C, 8, kT>(st, V, s, nrhs, x, y); break;
+        case 16: launch_spmv_pat_t<C, 16, kT>(st, V, s, nrhs, x, y); break;
+        case 32: launch_spmv_pat_t<C, 32, kT>(st, V, s, nrhs, x, y); break;
+        default: launch_spmv_pat_t<C, 0, false>(st, V, s, nrhs, x, y); break;
+    }
+}
+
 }  // namespace fe
 
 using namespace fe;
@@ -369,7 +486,18 @@ fe_status fe_spmv(fe_ctx* ctx, const fe_system* s, int32_t precision, int32_t nr
                                                                                   ((int64_t)m->n_act + 7) / 8));
     const int64_t n_items = (int64_t)m->n_act * nrhs;
     const unsigned col_blocks = (unsigned)((n_items + 255) / 256);
-    if (precision == FE_PREC_FP64) {
+    const void* terms = precision == FE_PREC_FP64 ? s->pat_t64.ptr
+                        : precision == FE_PREC_MIXED ? s->pat_t32.ptr
+                        : precision == FE_PREC_DF ? s->pat_tdf.ptr : nullptr;
+    const int64_t pat_blocks = ((int64_t)m->n_act + s->n_expl) * 3 * nrhs / 256 + 2;
+    if (s->n_pat && terms && pat_blocks < (1ll << 31)) {
+        if (precision == FE_PREC_FP64)
+            launch_spmv_pat<double2>(st, s, terms, nrhs, (const double2*)x, (double2*)y);
+        else if (precision == FE_PREC_MIXED)
+            launch_spmv_pat<float2>(st, s, terms, nrhs, (const float2*)x, (float2*)y);
+        else
+            launch_spmv_pat<float4>(st, s, terms, nrhs, (const float4*)x, (float4*)y);
+    } else if (precision == FE_PREC_FP64) {
         if (pow2 && nrhs >= 8)
             launch_spmm_rows<double2>(nrhs, st, ctx->num_sms, (const double2*)s->val64.ptr, s->stride, col, rp,
                                   (const double2*)x, (double2*)y, m->n_act);
