@@ -2,9 +2,15 @@
 //   b(W) = G(W, H_i) - int_Sext W . (n x curl H_i) ds,
 // with G the weak Engquist-Majda form of Eq. 3 (the same integrated-by-parts
 // form as the left-hand side) and H_i = p_hat H0 exp(-j k0 k_hat . r),
-// curl H_i = -j k0 k_hat x H_i.  One thread per (active node, wave) gathers
-// the outer faces around its node (2x2 Gauss points per face), so the sum is
-// deterministic and atomic-free.
+// curl H_i = -j k0 k_hat x H_i.  On an axis-aligned face the 2 x 2 Gauss sums
+// of a node's hat (or of its tangential gradient) times the wave's phase are
+// products of one-dimensional sums, so a first kernel tabulates those per
+// wave, axis and grid position (k_rhs_axis: eight phases each), and one thread
+// per (active node, wave) multiplies three table entries per face: a sine and
+// cosine in FP64 take this GPU some two hundred operations at a sixty-fourth
+// of the FP32 rate, and the direct sums needed sixteen pairs per face node
+// (719 us for 4 waves on 51^3 nodes).  The sums are deterministic and
+// atomic-free.
 #include "fe_internal.cuh"
 
 namespace fe {
@@ -14,74 +20,103 @@ struct Wave {
     double ar, ai;
 };
 
-__global__ void k_rhs(int nx, int ny, int nz, double hx, double hy, double hz, double ox, double oy, double oz,
-                      double k0, double sigma, const int* __restrict__ node_id, int n_act,
-                      const Wave* __restrict__ waves, int nrhs, unsigned abc, unsigned planes,
-                      const uint8_t* __restrict__ mat, int form_e, double2* __restrict__ B) {
+// One-dimensional sums of wave w at position i of an axis: over the (up to)
+// two elements beside it and two Gauss points each,
+//     val = sum (h/2) N e^{-j k0 k x},  grad = sum (h/2) N' e^{-j k0 k x},
+// and the phase at the position itself.
+struct AxisSum {
+    double2 val, grad, at;
+};
+
+__global__ void k_rhs_axis(int nx, int ny, int nz, double hx, double hy, double hz, double ox, double oy, double oz,
+                           double k0, const Wave* __restrict__ waves, int nrhs, AxisSum* __restrict__ tab) {
+    const int len = nx + ny + nz + 3;
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= (int64_t)len * nrhs) return;
+    const int w = (int)(t / len);
+    int i = (int)(t - (int64_t)w * len), axis = 0, n = nx;
+    double h = hx, org = ox;
+    if (i > nx) {
+        i -= nx + 1;
+        axis = 1;
+        n = ny;
+        h = hy;
+        org = oy;
+        if (i > ny) {
+            i -= ny + 1;
+            axis = 2;
+            n = nz;
+            h = hz;
+            org = oz;
+        }
+    }
+    const double k = waves[w].k[axis];
+    const double g0 = 0.5 - 0.5 / sqrt(3.0), g1 = 0.5 + 0.5 / sqrt(3.0);
+    AxisSum s;
+    s.val = s.grad = make_double2(0.0, 0.0);
+    for (int e = i - 1; e <= i; ++e) {
+        if (e < 0 || e >= n) continue;
+        const bool up = e == i - 1;  // the node is the element's upper end
+        for (int q = 0; q < 2; ++q) {
+            const double xi = q ? g1 : g0;
+            double sn, cs;
+            sincos(-k0 * k * (org + (e + xi) * h), &sn, &cs);
+            const double f = 0.5 * h * (up ? xi : 1.0 - xi), g = up ? 0.5 : -0.5;
+            s.val.x += f * cs;
+            s.val.y += f * sn;
+            s.grad.x += g * cs;
+            s.grad.y += g * sn;
+        }
+    }
+    sincos(-k0 * k * (org + i * h), &s.at.y, &s.at.x);
+    tab[t] = s;
+}
+
+__device__ __forceinline__ double2 zmul(double2 a, double2 b) {
+    return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+}
+
+__global__ void k_rhs(int nx, int ny, int nz, double k0, double sigma, const int* __restrict__ node_id, int n_act,
+                      const Wave* __restrict__ waves, const AxisSum* __restrict__ tab, int nrhs, unsigned abc,
+                      unsigned planes, const uint8_t* __restrict__ mat, int form_e, double2* __restrict__ B) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= (int64_t)n_act * nrhs) return;
     const int r = (int)(t / nrhs), w = (int)(t - (int64_t)r * nrhs);
     const int id = node_id[r];
     const int c[3] = {id % (nx + 1), (id / (nx + 1)) % (ny + 1), id / ((nx + 1) * (ny + 1))};
     const int dim[3] = {nx, ny, nz};
-    const double h[3] = {hx, hy, hz};
-    const double org[3] = {ox, oy, oz};
-    const Wave wv = waves[w];
     double br[3] = {0, 0, 0}, bi[3] = {0, 0, 0};
-    const double g0 = 0.5 - 0.5 / sqrt(3.0), g1 = 0.5 + 0.5 / sqrt(3.0);
-    for (int f = 0; f < 6; ++f) {
-        const int nu = f >> 1, side = f & 1;
-        if (c[nu] != (side ? dim[nu] : 0) || !((abc >> f) & 1u)) continue;  // absorbing faces only
-        const int t1 = nu == 0 ? 1 : 0, t2 = nu == 2 ? 1 : 2;
-        const double nsgn = side ? 1.0 : -1.0;
-        // n . k_hat and the element coordinate along the normal
-        const double nk = nsgn * wv.k[nu];
-        const int e_nu = side ? dim[nu] - 1 : 0;
-        for (int s2 = 0; s2 < 2; ++s2) {
-            const int e2 = c[t2] - 1 + s2;
-            if (e2 < 0 || e2 >= dim[t2]) continue;
-            for (int s1 = 0; s1 < 2; ++s1) {
-                const int e1 = c[t1] - 1 + s1;
-                if (e1 < 0 || e1 >= dim[t1]) continue;
-                const int a1 = c[t1] - e1, a2 = c[t2] - e2;  // local coordinates of the node
-                const double wq = 0.25 * h[t1] * h[t2];
-                for (int q = 0; q < 4; ++q) {
-                    const double xi1 = (q & 1) ? g1 : g0, xi2 = (q & 2) ? g1 : g0;
-                    const double f1 = a1 ? xi1 : 1.0 - xi1, f2 = a2 ? xi2 : 1.0 - xi2;
-                    const double N = f1 * f2;
-                    // tangential gradient of the hat, dotted with k_hat
-                    const double gk = (a1 ? 1.0 : -1.0) / h[t1] * f2 * wv.k[t1] +
-                                      (a2 ? 1.0 : -1.0) / h[t2] * f1 * wv.k[t2];
-                    double x[3];
-                    x[nu] = org[nu] + (e_nu + side) * h[nu];
-                    x[t1] = org[t1] + (e1 + xi1) * h[t1];
-                    x[t2] = org[t2] + (e2 + xi2) * h[t2];
-                    const double ph = -k0 * (wv.k[0] * x[0] + wv.k[1] * x[1] + wv.k[2] * x[2]);
-                    double sn, cs;
-                    sincos(ph, &sn, &cs);
-                    // phase factor times amplitude
-                    const double er = wv.ar * cs - wv.ai * sn, ei = wv.ar * sn + wv.ai * cs;
-                    double hr[3], hi[3];
-                    for (int d = 0; d < 3; ++d) {
-                        hr[d] = wv.p[d] * er;
-                        hi[d] = wv.p[d] * ei;
-                    }
-                    const double nhr = nsgn * hr[nu], nhi = nsgn * hi[nu];  // n . H_i
-                    for (int al = 0; al < 3; ++al) {
-                        // n x curl H_i = -j k0 (k_hat (n.H_i) - H_i (n.k_hat))
-                        const double ur = wv.k[al] * nhr - hr[al] * nk, ui = wv.k[al] * nhi - hi[al] * nk;
-                        // -N (n x curl H_i) = j k0 N u = k0 N (-ui + j ur)
-                        double vr = -N * k0 * ui, vi = N * k0 * ur;
-                        if (al != nu) {
-                            // j k0 N H_al + sigma (j / 2k0)(grad_t N . (-j k0 k_t)) H_al
-                            //   = j k0 N H_al + (sigma / 2)(grad_t N . k_hat) H_al
-                            vr += -k0 * N * hi[al] + 0.5 * sigma * gk * hr[al];
-                            vi += k0 * N * hr[al] + 0.5 * sigma * gk * hi[al];
-                        }
-                        br[al] += wq * vr;
-                        bi[al] += wq * vi;
-                    }
+    if (c[0] == 0 || c[0] == nx || c[1] == 0 || c[1] == ny || c[2] == 0 || c[2] == nz) {
+        const Wave wv = waves[w];
+        const AxisSum* tw = tab + (size_t)w * (nx + ny + nz + 3);
+        const int first[3] = {0, nx + 1, nx + ny + 2};
+#pragma unroll
+        for (int f = 0; f < 6; ++f) {
+            const int nu = f >> 1, side = f & 1;
+            if (c[nu] != (side ? dim[nu] : 0) || !((abc >> f) & 1u)) continue;  // absorbing faces only
+            const int t1 = nu == 0 ? 1 : 0, t2 = nu == 2 ? 1 : 2;
+            const AxisSum& a1 = tw[first[t1] + c[t1]];
+            const AxisSum& a2 = tw[first[t2] + c[t2]];
+            const double2 e = zmul(make_double2(wv.ar, wv.ai), tw[first[nu] + c[nu]].at);
+            const double2 v1 = zmul(a1.val, e);
+            const double2 val = zmul(v1, a2.val);                    // int N e^{-j k0 k.r}
+            const double2 d1 = zmul(zmul(a1.grad, e), a2.val), d2 = zmul(v1, a2.grad);
+            const double gr = wv.k[t1] * d1.x + wv.k[t2] * d2.x;     // int (grad_t N . k_hat) e^{-j k0 k.r}
+            const double gi = wv.k[t1] * d1.y + wv.k[t2] * d2.y;
+            const double nsgn = side ? 1.0 : -1.0;
+            const double nk = nsgn * wv.k[nu], np = nsgn * wv.p[nu];  // n . k_hat, n . p_hat
+#pragma unroll
+            for (int al = 0; al < 3; ++al) {
+                // -N (n x curl H_i) = j k0 N (k_hat (n.H_i) - H_i (n.k_hat)), and for the tangential
+                // components j k0 N H_al + sigma (j / 2k0)(grad_t N . (-j k0 k_t)) H_al
+                double u = wv.k[al] * np - wv.p[al] * nk;
+                if (al != nu) {
+                    u += wv.p[al];
+                    br[al] += 0.5 * sigma * wv.p[al] * gr;
+                    bi[al] += 0.5 * sigma * wv.p[al] * gi;
                 }
+                br[al] -= k0 * u * val.y;
+                bi[al] += k0 * u * val.x;
             }
         }
     }
@@ -105,13 +140,20 @@ fe_status build_rhs(fe_ctx* ctx, const fe_system* s, int nrhs, const fe_planewav
         hw[w].ar = waves[w].amplitude.re;
         hw[w].ai = waves[w].amplitude.im;
     }
-    FE_TRY(dev_alloc(st, wave_buf, (size_t)nrhs * sizeof(Wave)));
+    // the waves, then the axis tables (16-byte aligned behind them)
+    const int len = m->nx + m->ny + m->nz + 3;
+    const size_t tab_at = ((size_t)nrhs * sizeof(Wave) + 15) & ~(size_t)15;
+    FE_TRY(dev_alloc(st, wave_buf, tab_at + (size_t)nrhs * len * sizeof(AxisSum)));
     FE_CUDA(cudaMemcpyAsync(wave_buf.ptr, hw.data(), (size_t)nrhs * sizeof(Wave), cudaMemcpyHostToDevice, st));
+    AxisSum* tab = (AxisSum*)((char*)wave_buf.ptr + tab_at);
+    k_rhs_axis<<<(unsigned)(((int64_t)len * nrhs + 63) / 64), 64, 0, st>>>(
+        m->nx, m->ny, m->nz, m->h[0], m->h[1], m->h[2], m->origin[0], m->origin[1], m->origin[2], s->k0,
+        (const Wave*)wave_buf.ptr, nrhs, tab);
+    FE_LAUNCHED();
     const int64_t n = (int64_t)m->n_act * nrhs;
-    k_rhs<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(m->nx, m->ny, m->nz, m->h[0], m->h[1], m->h[2],
-                                                       m->origin[0], m->origin[1], m->origin[2], s->k0, s->sigma,
+    k_rhs<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(m->nx, m->ny, m->nz, s->k0, s->sigma,
                                                        (const int*)m->node_id.ptr, m->n_act,
-                                                       (const Wave*)wave_buf.ptr, nrhs, abc_faces(m->boundary),
+                                                       (const Wave*)wave_buf.ptr, tab, nrhs, abc_faces(m->boundary),
                                                        pack_planes(m->boundary), (const uint8_t*)m->material.ptr,
                                                        s->formulation == FE_FORMULATION_E ? 1 : 0, d_B);
     FE_LAUNCHED();
