@@ -630,7 +630,7 @@ fe_status fe_system_info(const fe_system* s, fe_system_stats* out) {
     int64_t bytes = 0;
     for (const DevBuf* b : {&s->tables, &s->val64, &s->val32, &s->valdf, &s->dinv64, &s->dinv32, &s->dinvdf,
                             &s->row_class, &s->stencil, &s->cost_prefix, &s->cost_prefix_alu, &s->expl_prefix,
-                            &s->dict_idx, &s->dict_vals, &s->pat_first, &s->pat_id, &s->pat_tab, &s->pat_t64,
+                            &s->dict_idx, &s->dict_vals, &s->pat_first, &s->pat_id, &s->pat_row, &s->pat_tab, &s->pat_t64,
                             &s->pat_t32, &s->pat_tdf, &s->pat_cost, &s->pat_list, &s->bicp_l, &s->bicp_linv,
                              &s->bicp_tpos, &s->bicp_tab, &s->bicp_lev, &s->bicp_nlev})
         bytes += (int64_t)b->bytes;

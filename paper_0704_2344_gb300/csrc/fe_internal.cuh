@@ -194,6 +194,7 @@ struct fe_system {
     int64_t pat_cost_total = 0;
     fe::DevBuf pat_first;                // int [n_pat]: first row of each pattern
     fe::DevBuf pat_id;               // uint16 [n_act]
+    fe::DevBuf pat_row;              // int4 [n_act]: (first term, steps and kind, grid node, pattern)
     fe::DevBuf pat_tab;              // int4 [n_pat]: (first term triple, n_re, n_im, real diagonal blocks)
     fe::DevBuf pat_t64, pat_t32, pat_tdf;  // terms [n_pat * kPatStride * 3]: double2 / float2 / float4
     fe::DevBuf pat_cost;             // int [n_act + 1]: prefix sum of the rows' product cost

@@ -282,7 +282,8 @@ __global__ void __launch_bounds__(256) k_pat_spread(const int* __restrict__ grou
                                                     int64_t stride, int n, double2* __restrict__ val64,
                                                     float2* __restrict__ val32, float4* __restrict__ valdf,
                                                     double2* __restrict__ dinv64, float2* __restrict__ dinv32,
-                                                    float4* __restrict__ dinvdf, uint16_t* __restrict__ pat_id,
+                                                    float4* __restrict__ dinvdf, const int* __restrict__ node_id,
+                                                    uint16_t* __restrict__ pat_id, int4* __restrict__ pat_row,
                                                     int* __restrict__ cost, int* __restrict__ expl) {
     const int r = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
     if (r >= n) return;
@@ -304,6 +305,7 @@ __global__ void __launch_bounds__(256) k_pat_spread(const int* __restrict__ grou
     if (lane == 0) {
         const int4 t = __ldg(tab + id);
         pat_id[r] = (uint16_t)id;
+        pat_row[r] = make_int4(3 * t.x, t.y | t.z << 10 | t.w << 20, __ldg(node_id + r), id);
         cost[r] = pattern_cost(t.y, t.z, t.w != 0);
         expl[r] = t.w ? 0 : 1;
     }
@@ -384,6 +386,7 @@ fe_status build_patterns(fe_ctx* ctx, fe_system* s, const DevBuf& row_group, int
     fe_status e;
     const size_t triples = (size_t)n_pat * kPatStride;
     if ((e = dev_alloc(st, s->pat_id, (size_t)n * sizeof(uint16_t))) != FE_OK) return done(e);
+    if ((e = dev_alloc(st, s->pat_row, (size_t)n * sizeof(int4))) != FE_OK) return done(e);
     if ((e = dev_alloc(st, s->pat_tab, (size_t)n_pat * sizeof(int4))) != FE_OK) return done(e);
     if ((e = dev_alloc(st, s->pat_t64, triples * 3 * sizeof(double2))) != FE_OK) return done(e);
     if (s->val32.ptr && (e = dev_alloc(st, s->pat_t32, triples * 3 * sizeof(float2))) != FE_OK) return done(e);
@@ -404,7 +407,7 @@ fe_status build_patterns(fe_ctx* ctx, fe_system* s, const DevBuf& row_group, int
     k_pat_spread<<<(unsigned)(((int64_t)n * 32 + 255) / 256), 256, 0, st>>>(
         (const int*)row_group.ptr, first, (const int4*)s->pat_tab.ptr, rp, s->stride, n, (double2*)s->val64.ptr,
         (float2*)s->val32.ptr, (float4*)s->valdf.ptr, (double2*)s->dinv64.ptr, (float2*)s->dinv32.ptr,
-        (float4*)s->dinvdf.ptr, (uint16_t*)s->pat_id.ptr, cost, (int*)expl.ptr);
+        (float4*)s->dinvdf.ptr, (const int*)m->node_id.ptr, (uint16_t*)s->pat_id.ptr, (int4*)s->pat_row.ptr, cost, (int*)expl.ptr);
     count_launches(2);
     if ((e = scan_exclusive(st, cost, cost, n, d_totals, ctx->scan_tmp)) != FE_OK) return done(e);
     cudaMemcpyAsync(cost + n, d_totals, sizeof(int), cudaMemcpyDeviceToDevice, st);
@@ -424,7 +427,7 @@ fe_status build_patterns(fe_ctx* ctx, fe_system* s, const DevBuf& row_group, int
 
 void drop_patterns(fe_system* s) {
     cudaStream_t st = s->ctx->stream;
-    for (DevBuf* b : {&s->pat_first, &s->pat_id, &s->pat_tab, &s->pat_t64, &s->pat_t32, &s->pat_tdf, &s->pat_cost,
+    for (DevBuf* b : {&s->pat_first, &s->pat_id, &s->pat_row, &s->pat_tab, &s->pat_t64, &s->pat_t32, &s->pat_tdf, &s->pat_cost,
                       &s->pat_list})
         dev_free(st, *b);
     s->n_pat = 0;

@@ -60,7 +60,10 @@ struct TermAcc {
         re -= t.x * x.y;
         im += t.x * x.x;
     }
-    __device__ __forceinline__ C result() const { return mk(re, im); }
+    __device__ __forceinline__ void add(const TermAcc& o) {
+        re += o.re;
+        im += o.im;
+    }
     __device__ __forceinline__ C result_norm() { return mk(re, im); }
 };
 template <>
@@ -74,7 +77,10 @@ struct TermAcc<float4> {
         df_mac(a[0], a[1], -t.x, -t.y, x.y, x.w);
         df_mac(a[2], a[3], t.x, t.y, x.x, x.z);
     }
-    __device__ __forceinline__ float4 result() const { return df_result(a); }
+    __device__ __forceinline__ void add(const TermAcc& o) {
+        df_add(a[0], a[1], o.a[0], o.a[1]);
+        df_add(a[2], a[3], o.a[2], o.a[3]);
+    }
     __device__ __forceinline__ float4 result_norm() { return df_result_norm(a); }
 };
 
@@ -99,17 +105,45 @@ __device__ __forceinline__ void acc_butterfly(TermAcc<C>& acc, int o) {
 template <typename C, typename Base, typename Load>
 __device__ __forceinline__ void pattern_terms(TermAcc<C>& acc, const C* terms, int n_re, int n_im, int R, int c,
                                               Base&& base, Load&& load) {
+    auto entry = [&](int code) { return load((size_t)(base(code_line(code)) + code_delta(code)) * R + c); };
+    if constexpr (std::is_same<C, float4>::value) {
+        // FP32 pairs: two accumulators, every other term each, so that a warp
+        // does not wait for one chain of additions (2 to 4 % of an iteration;
+        // FP64 and complex64, with one operation per term and part, lose by it)
+        TermAcc<C> other;
+        int t = 0;
+        for (; t + 4 <= n_re; t += 4) {
+            C q[4], x[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                q[k] = terms[3 * (t + k)];
+                x[k] = entry(term_code(q[k]));
+            }
+            acc.add_re(q[0], x[0]);
+            other.add_re(q[1], x[1]);
+            acc.add_re(q[2], x[2]);
+            other.add_re(q[3], x[3]);
+        }
+        for (; t < n_re; ++t) {
+            const C q = terms[3 * t];
+            acc.add_re(q, entry(term_code(q)));
+        }
+        for (; t < n_re + n_im; ++t) {
+            const C q = terms[3 * t];
+            other.add_im(q, entry(term_code(q)));
+        }
+        acc.add(other);
+    } else {
 #pragma unroll 3
-    for (int t = 0; t < n_re; ++t) {
-        const C q = terms[3 * t];
-        const int code = term_code(q);
-        acc.add_re(q, load((size_t)(base(code_line(code)) + code_delta(code)) * R + c));
-    }
-    terms += 3 * n_re;
-    for (int t = 0; t < n_im; ++t) {
-        const C q = terms[3 * t];
-        const int code = term_code(q);
-        acc.add_im(q, load((size_t)(base(code_line(code)) + code_delta(code)) * R + c));
+        for (int t = 0; t < n_re; ++t) {
+            const C q = terms[3 * t];
+            acc.add_re(q, entry(term_code(q)));
+        }
+        terms += 3 * n_re;
+        for (int t = 0; t < n_im; ++t) {
+            const C q = terms[3 * t];
+            acc.add_im(q, entry(term_code(q)));
+        }
     }
 }
 
@@ -136,9 +170,28 @@ __device__ __forceinline__ void pattern_diag(TermAcc<C>& acc, const C* terms, in
 #pragma unroll 2
         for (int k = 0; k < 8; ++k) line(k + (k >= 4), false);
         line(4, true);
-    } else {
+    } else if constexpr (!std::is_same<C, float4>::value) {
 #pragma unroll 3
         for (int m = 0; m < 9; ++m) line(m, false);
+    } else {
+        // the lines below the row's plane in one accumulator, those above in
+        // another, the row's own plane split between them
+        TermAcc<C> other;
+        auto both = [&](int m, int k) {
+            const size_t i = (size_t)(base(m) + al) * R + c, j = (size_t)(base(k) + al) * R + c;
+            const C x0 = load(i - 3 * R), x1 = load(i), x2 = load(i + 3 * R);
+            const C z0 = load(j - 3 * R), z1 = load(j), z2 = load(j + 3 * R);
+            acc.add_re(terms[9 * m], x0);
+            other.add_re(terms[9 * k], z0);
+            acc.add_re(terms[9 * m + 3], x1);
+            other.add_re(terms[9 * k + 3], z1);
+            acc.add_re(terms[9 * m + 6], x2);
+            other.add_re(terms[9 * k + 6], z2);
+        };
+#pragma unroll 2
+        for (int m = 0; m < 4; ++m) both(m, 8 - m);
+        line(4, false);
+        acc.add(other);
     }
 }
 
@@ -146,6 +199,7 @@ __device__ __forceinline__ void pattern_diag(TermAcc<C>& acc, const C* terms, in
 template <typename C>
 struct PatView {
     const uint16_t* id;    // [n_rows] pattern of each row
+    const int4* row;       // [n_rows] (first term, n_re | n_im << 10 | real diagonal blocks << 20, grid node, pattern)
     const int4* tab;       // [n_pat] (first term triple, n_re, n_im, 1: real diagonal blocks)
     const C* terms;
     const int* node_id;    // [n_rows] grid node of each row

@@ -112,7 +112,7 @@ int64_t estimate_bytes(const fe_mesh_desc& d, int nrhs, int width, int prec, int
     const int64_t per_entry = prec == FE_PREC_FP64 ? 16 : (prec == FE_PREC_MIXED ? 24 : 32);
     const int64_t sys = 9 * stride * per_entry + 9 * nodes * 24 + nodes * 13 + 65536;
     // row patterns: term lists, the row tables and what their construction holds
-    const int64_t pat = (int64_t)pat_limit(nodes) * kPatStride * 3 * per_entry + 64 * nodes + (1 << 18);
+    const int64_t pat = (int64_t)pat_limit(nodes) * kPatStride * 3 * per_entry + 80 * nodes + (1 << 18);
     const int64_t rhs = 3 * nodes * (int64_t)nrhs * 16;
     // the packed explicit rows of a single-column launch: at most every block
     const int64_t pk = (width == 1 && prec != FE_PREC_FP64) ? 9 * nnzb : 0;

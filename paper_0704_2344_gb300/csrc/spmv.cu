@@ -349,77 +349,175 @@ static void launch_spmv_warp(int R, unsigned blocks, cudaStream_t st, const C* v
     }
 }
 
-// y = A x from the row patterns, R columns (R = 0: nrhs of them).  The matrix
-// is a few hundred kilobytes of terms that stay in L1 and L2, so the product
-// moves the vectors and the row tables only: the 80^3 aircraft's complex64
-// product reads 25 MB of vectors instead of 1.1 GB of blocks.
-// One thread per (row, component, column), so that the lanes of a warp read
-// consecutive vector entries; the first blocks take the explicit rows
-// (collected in a list, so that a warp holds rows of like length), the others
-// sweep all rows for the real diagonal ones.  kTile (complex64, R >= 8): the
-// sweep takes four consecutive rows per thread, which share two of every
-// three vector entries along a grid line; the product is then bound by the L1
-// traffic of those entries.
-template <typename C, int R_, bool kTile>
+// ---------------------------------------------------------------------------
+// y = A x from the row patterns.  The matrix is a few hundred kilobytes of
+// terms that stay in L1 and L2, so a product moves the vectors and the row
+// tables only: the 80^3 aircraft's complex64 product reads 25 MB of vectors
+// and tables instead of 1.1 GB of blocks.  Work items are (row, component,
+// column), consecutive lanes taking consecutive vector entries.  Four forms:
+//
+//   split   few items (below kSplitItems): 2 to 8 lanes share one, so that the
+//           chip's lanes are used and a lane's chain of dependent loads is short;
+//   plain   one lane per item; the first blocks take the explicit rows
+//           (collected in a list, so that a warp holds rows of like length),
+//           the others sweep all rows for the real diagonal ones.  FP64 and
+//           FP32 pairs, which are bound by their arithmetic;
+//   keep    complex64, 1, 2 or 4 columns: one CTA per SM walks a range of
+//           rows, every thread staying on one component and column, with the
+//           27 weights of its pattern in registers;
+//   tile    complex64, 8, 16 or 32 columns: the same walk with four
+//           consecutive rows per thread, which share two of every three
+//           entries along a grid line.  Walking a range keeps a row's lines in
+//           L1 for the rows above and beside it.
+// ---------------------------------------------------------------------------
+template <typename C, int R_>
+__device__ __forceinline__ void pat_item(const PatView<C>& V, const C* __restrict__ x, C* __restrict__ y, int row,
+                                         int al, int R, int c, bool want_diag) {
+    const int4 t = __ldg(V.row + row);
+    if (((t.y >> 20) & 1) != (int)want_diag) return;
+    const LineRanks base{V.node_rank + t.z, V.sy, V.sz};
+    const C* terms = V.terms + t.x + al;
+    auto load = [&](size_t i) { return __ldg(x + i); };
+    TermAcc<C> acc;
+    if (want_diag) pattern_diag<C, true>(acc, terms, al, R, c, base, load);
+    else pattern_terms<C>(acc, terms, t.y & 0x3ff, (t.y >> 10) & 0x3ff, R, c, base, load);
+    y[((size_t)3 * row + al) * R + c] = acc.result_norm();
+}
+
+template <typename C, int R_>
 __global__ void __launch_bounds__(256) k_spmv_pat(PatView<C> V, int n_rows, const int* __restrict__ list, int n_expl,
                                                   int expl_blocks, int nrhs, const C* __restrict__ x,
                                                   C* __restrict__ y) {
     const int R = R_ ? R_ : nrhs;
-    auto load = [&](size_t i) { return __ldg(x + i); };
-    if ((int)blockIdx.x < expl_blocks) {
-        const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-        const int64_t d = e / R;
-        const int c = (int)(e - d * R), i = (int)(d / 3), al = (int)(d - 3 * (int64_t)i);
-        if (i >= n_expl) return;
-        const int row = __ldg(list + i);
-        const int4 t = __ldg(V.tab + __ldg(V.id + row));
-        const LineRanks base{V.node_rank + __ldg(V.node_id + row), V.sy, V.sz};
-        TermAcc<C> acc;
-        pattern_terms<C>(acc, V.terms + (size_t)t.x * 3 + al, t.y, t.z, R, c, base, load);
-        y[((size_t)3 * row + al) * R + c] = acc.result_norm();
-        return;
-    }
-    const int64_t e = (int64_t)(blockIdx.x - expl_blocks) * blockDim.x + threadIdx.x;
+    const bool expl = (int)blockIdx.x < expl_blocks;
+    const int64_t e = (int64_t)(expl ? blockIdx.x : blockIdx.x - expl_blocks) * blockDim.x + threadIdx.x;
     const int64_t d = e / R;
-    const int c = (int)(e - d * R);
-    auto one_row = [&](int row, int al) {
-        const int4 t = __ldg(V.tab + __ldg(V.id + row));
-        if (!t.w) return;
+    const int c = (int)(e - d * R), i = (int)(d / 3), al = (int)(d - 3 * (int64_t)i);
+    if (i >= (expl ? n_expl : n_rows)) return;
+    if (expl) pat_item<C, R_>(V, x, y, __ldg(list + i), al, R, c, false);
+    else pat_item<C, R_>(V, x, y, i, al, R, c, true);
+}
+
+// split: K lanes per item, K R columns (a power of two up to 32) per warp part.
+template <typename C, int R, int K>
+__global__ void __launch_bounds__(256) k_spmv_pat_split(PatView<C> V, int n_rows, const C* __restrict__ x,
+                                                        C* __restrict__ y) {
+    const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int c = (int)(t0 % R), part = (int)(t0 / R) % K;
+    const int64_t d = t0 / (R * K);
+    const int row = (int)(d / 3), al = (int)(d - 3 * (int64_t)row);
+    const bool on = row < n_rows;
+    TermAcc<C> acc;
+    if (on) {
+        const int4 t = __ldg(V.row + row);
+        const LineRanks base{V.node_rank + t.z, V.sy, V.sz};
+        const C* terms = V.terms + t.x + al;
+        const int n_re = t.y & 0x3ff, n_im = (t.y >> 10) & 0x3ff;
+#pragma unroll 4
+        for (int k = part; k < n_re; k += K) {
+            const C q = terms[3 * k];
+            const int code = term_code(q);
+            acc.add_re(q, __ldg(x + (size_t)(base(code_line(code)) + code_delta(code)) * R + c));
+        }
+        for (int k = n_re + part; k < n_re + n_im; k += K) {
+            const C q = terms[3 * k];
+            const int code = term_code(q);
+            acc.add_im(q, __ldg(x + (size_t)(base(code_line(code)) + code_delta(code)) * R + c));
+        }
+    }
+#pragma unroll
+    for (int o = R; o < R * K; o <<= 1) acc_butterfly(acc, o);
+    if (on && part == 0) y[((size_t)3 * row + al) * R + c] = acc.result_norm();
+}
+
+// keep: a thread's component and column do not change along its walk, since
+// the block's threads are a multiple of 3 R.
+constexpr int kKeepThreads = 768;
+template <int R>
+__global__ void __launch_bounds__(kKeepThreads, 1) k_spmv_pat_keep(PatView<float2> V, int n_rows,
+                                                                  const int* __restrict__ list, int n_expl,
+                                                                  const float2* __restrict__ x,
+                                                                  float2* __restrict__ y) {
+    static_assert(kKeepThreads % (3 * R) == 0, "a thread keeps its component and column");
+    const int c = threadIdx.x % R, al = (threadIdx.x / R) % 3, step = kKeepThreads / (3 * R);
+    // explicit rows of this block, one walk beside the other
+    const int e0 = (int)((int64_t)blockIdx.x * n_expl / gridDim.x), e1 = (int)((int64_t)(blockIdx.x + 1) * n_expl / gridDim.x);
+    for (int i = e0 + (int)threadIdx.x / (3 * R); i < e1; i += step)
+        pat_item<float2, R>(V, x, y, __ldg(list + i), al, R, c, false);
+    const int r0 = (int)((int64_t)blockIdx.x * n_rows / gridDim.x), r1 = (int)((int64_t)(blockIdx.x + 1) * n_rows / gridDim.x);
+    float w[27];
+    int held = -1;
+    for (int row = r0 + (int)threadIdx.x / (3 * R); row < r1; row += step) {
+        const int id = __ldg(V.id + row);
+        const int4 t = __ldg(V.tab + id);
+        if (!t.w) continue;
+        if (id != held) {
+#pragma unroll
+            for (int k = 0; k < 27; ++k) w[k] = __ldg(&V.terms[(size_t)t.x * 3 + al + 3 * k].x);
+            held = id;
+        }
         const LineRanks base{V.node_rank + __ldg(V.node_id + row), V.sy, V.sz};
-        TermAcc<C> acc;
-        pattern_diag<C, true>(acc, V.terms + (size_t)t.x * 3 + al, al, R, c, base, load);
-        y[((size_t)3 * row + al) * R + c] = acc.result_norm();
-    };
-    if constexpr (!kTile) {
-        const int row = (int)(d / 3);
-        if (row < n_rows) one_row(row, (int)(d - 3 * (int64_t)row));
-    } else {
-        const int r0 = 4 * (int)(d / 3), al = (int)(d % 3);
-        if (r0 >= n_rows) return;
+        float re = 0.f, im = 0.f, cr = 0.f, ci = 0.f;
+#pragma unroll
+        for (int m = 0; m < 9; ++m) {
+            const float2* xp = x + (size_t)(base(m) + al) * R + c;
+            const float2 x0 = __ldg(xp - 3 * R), x1 = __ldg(xp), x2 = __ldg(xp + 3 * R);
+            re += w[3 * m] * x0.x;
+            im += w[3 * m] * x0.y;
+            if (m == 4) {  // the row's own entry last
+                cr = w[13] * x1.x;
+                ci = w[13] * x1.y;
+            } else {
+                re += w[3 * m + 1] * x1.x;
+                im += w[3 * m + 1] * x1.y;
+            }
+            re += w[3 * m + 2] * x2.x;
+            im += w[3 * m + 2] * x2.y;
+        }
+        y[((size_t)3 * row + al) * R + c] = make_float2(re + cr, im + ci);
+    }
+}
+
+// tile: (four rows, component, column) per thread.
+constexpr int kTileThreads = 1024;
+template <int R>
+__global__ void __launch_bounds__(kTileThreads, 1) k_spmv_pat_tile(PatView<float2> V, int n_rows,
+                                                                  const int* __restrict__ list, int n_expl,
+                                                                  const float2* __restrict__ x,
+                                                                  float2* __restrict__ y) {
+    const int e0 = (int)((int64_t)blockIdx.x * n_expl / gridDim.x), e1 = (int)((int64_t)(blockIdx.x + 1) * n_expl / gridDim.x);
+    for (int q = threadIdx.x; q < (e1 - e0) * 3 * R; q += kTileThreads) {
+        const int c = q % R, d = q / R;
+        pat_item<float2, R>(V, x, y, __ldg(list + e0 + d / 3), d % 3, R, c, false);
+    }
+    const int n4 = (n_rows + 3) / 4;
+    const int q0 = (int)((int64_t)blockIdx.x * n4 / gridDim.x), q1 = (int)((int64_t)(blockIdx.x + 1) * n4 / gridDim.x);
+    for (int q = threadIdx.x; q < (q1 - q0) * 3 * R; q += kTileThreads) {
+        const int c = q % R, d = q / R, al = d % 3, r0 = 4 * (q0 + d / 3);
         const int id0 = __ldg(V.id + r0);
         bool tile = r0 + 3 < n_rows;
         if (tile)
             tile = __ldg(V.id + r0 + 1) == id0 && __ldg(V.id + r0 + 2) == id0 && __ldg(V.id + r0 + 3) == id0 &&
                    __ldg(V.node_id + r0 + 3) - __ldg(V.node_id + r0) == 3;
-        const int4 t = __ldg(V.tab + id0);
-        if (tile && !t.w) return;
         if (!tile) {
-            for (int row = r0; row < min(r0 + 4, n_rows); ++row) one_row(row, al);
-            return;
+            for (int row = r0; row < min(r0 + 4, n_rows); ++row) pat_item<float2, R>(V, x, y, row, al, R, c, true);
+            continue;
         }
-        const C* terms = V.terms + (size_t)t.x * 3 + al;
+        const int4 t = __ldg(V.tab + id0);
+        if (!t.w) continue;
+        const float2* terms = V.terms + (size_t)t.x * 3 + al;
         const LineRanks base{V.node_rank + __ldg(V.node_id + r0), V.sy, V.sz};
-        TermAcc<C> acc[4];
-        C own[4];
+        TermAcc<float2> acc[4];
+        float2 own[4];
         auto line = [&](int m, bool centre) {
-            const C* xp = x + ((size_t)(base(m) + al) * R + c) - 3 * R;
-            C v[6];
+            const float2* xp = x + ((size_t)(base(m) + al) * R + c) - 3 * R;
+            float2 v[6];
 #pragma unroll
             for (int k = 0; k < 6; ++k) v[k] = __ldg(xp + 3 * k * R);
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
                 if (centre && k == 1) continue;
-                const C w = __ldg(terms + 9 * m + 3 * k);
+                const float2 w = __ldg(terms + 9 * m + 3 * k);
 #pragma unroll
                 for (int j = 0; j < 4; ++j) acc[j].add_re(w, v[j + k]);
             }
@@ -430,7 +528,7 @@ __global__ void __launch_bounds__(256) k_spmv_pat(PatView<C> V, int n_rows, cons
 #pragma unroll 2
         for (int k = 0; k < 8; ++k) line(k + (k >= 4), false);
         line(4, true);  // the rows' own entries last
-        const C w = __ldg(terms + 39);
+        const float2 w = __ldg(terms + 39);
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[j].add_re(w, own[j]);
 #pragma unroll
@@ -438,31 +536,66 @@ __global__ void __launch_bounds__(256) k_spmv_pat(PatView<C> V, int n_rows, cons
     }
 }
 
-template <typename C, int R, bool kTile>
-static void launch_spmv_pat_t(cudaStream_t st, const PatView<C>& V, const fe_system* s, int nrhs, const C* x, C* y) {
+// Items below which lanes share them: about half of the chip's resident
+// threads (152 SMs x 2048); items from which the walks, with one or a quarter
+// of an item per lane and step, have work for their 117 000 or 156 000 lanes.
+constexpr int64_t kSplitItems = 150000, kKeepItems = 300000, kTileItems = 600000;
+
+template <typename C, int R>
+static void launch_pat_plain(cudaStream_t st, const PatView<C>& V, const fe_system* s, int nrhs, const C* x, C* y) {
+    const int64_t expl = ((int64_t)s->n_expl * 3 * nrhs + 255) / 256, all = ((int64_t)s->mesh->n_act * 3 * nrhs + 255) / 256;
+    k_spmv_pat<C, R><<<(unsigned)(expl + all), 256, 0, st>>>(V, s->mesh->n_act, (const int*)s->pat_list.ptr, s->n_expl,
+                                                            (int)expl, nrhs, x, y);
+}
+
+template <typename C, int R>
+static void launch_pat_r(cudaStream_t st, const PatView<C>& V, const fe_system* s, int sms, const C* x, C* y) {
     const int n = s->mesh->n_act;
-    const int64_t expl = ((int64_t)s->n_expl * 3 * nrhs + 255) / 256;
-    const int64_t rows = kTile ? ((int64_t)n + 3) / 4 : n;
-    const int64_t all = (rows * 3 * nrhs + 255) / 256;
-    k_spmv_pat<C, R, kTile><<<(unsigned)(expl + all), 256, 0, st>>>(V, n, (const int*)s->pat_list.ptr, s->n_expl,
-                                                                   (int)expl, nrhs, x, y);
+    const int64_t items = (int64_t)n * 3 * R;
+    auto blocks = [&](int k) { return (unsigned)((items * k + 255) / 256); };
+    if constexpr (8 * R <= 32)
+        if (8 * items <= 2 * kSplitItems) {
+            k_spmv_pat_split<C, R, 8><<<blocks(8), 256, 0, st>>>(V, n, x, y);
+            return;
+        }
+    if constexpr (4 * R <= 32)
+        if (4 * items <= 2 * kSplitItems) {
+            k_spmv_pat_split<C, R, 4><<<blocks(4), 256, 0, st>>>(V, n, x, y);
+            return;
+        }
+    if constexpr (2 * R <= 32)
+        if (items <= kSplitItems) {
+            k_spmv_pat_split<C, R, 2><<<blocks(2), 256, 0, st>>>(V, n, x, y);
+            return;
+        }
+    if constexpr (std::is_same<C, float2>::value && R <= 4)
+        if (items >= kKeepItems) {
+            k_spmv_pat_keep<R><<<sms, kKeepThreads, 0, st>>>(V, n, (const int*)s->pat_list.ptr, s->n_expl, x, y);
+            return;
+        }
+    if constexpr (std::is_same<C, float2>::value && R >= 8)
+        if (items >= kTileItems) {
+            k_spmv_pat_tile<R><<<sms, kTileThreads, 0, st>>>(V, n, (const int*)s->pat_list.ptr, s->n_expl, x, y);
+            return;
+        }
+    launch_pat_plain<C, R>(st, V, s, R, x, y);
 }
 
 template <typename C>
-static void launch_spmv_pat(cudaStream_t st, const fe_system* s, const void* terms, int nrhs, const C* x, C* y) {
+static void launch_spmv_pat(cudaStream_t st, const fe_system* s, int sms, const void* terms, int nrhs, const C* x,
+                            C* y) {
     const fe_mesh* m = s->mesh;
-    const PatView<C> V{(const uint16_t*)s->pat_id.ptr, (const int4*)s->pat_tab.ptr, (const C*)terms,
+    const PatView<C> V{(const uint16_t*)s->pat_id.ptr, (const int4*)s->pat_row.ptr, (const int4*)s->pat_tab.ptr, (const C*)terms,
                        (const int*)m->node_id.ptr,     (const int*)m->node_rank.ptr, m->nx + 1,
                        (m->nx + 1) * (m->ny + 1)};
-    constexpr bool kT = std::is_same<C, float2>::value;
     switch (nrhs) {
-        case 1: launch_spmv_pat_t<C, 1, false>(st, V, s, nrhs, x, y); break;
-        case 2: launch_spmv_pat_t<C, 2, false>(st, V, s, nrhs, x, y); break;
-        case 4: launch_spmv_pat_t<C, 4, false>(st, V, s, nrhs, x, y); break;
-        case 8: launch_spmv_pat_t<C, 8, kT>(st, V, s, nrhs, x, y); break;
-        case 16: launch_spmv_pat_t<C, 16, kT>(st, V, s, nrhs, x, y); break;
-        case 32: launch_spmv_pat_t<C, 32, kT>(st, V, s, nrhs, x, y); break;
-        default: launch_spmv_pat_t<C, 0, false>(st, V, s, nrhs, x, y); break;
+        case 1: launch_pat_r<C, 1>(st, V, s, sms, x, y); break;
+        case 2: launch_pat_r<C, 2>(st, V, s, sms, x, y); break;
+        case 4: launch_pat_r<C, 4>(st, V, s, sms, x, y); break;
+        case 8: launch_pat_r<C, 8>(st, V, s, sms, x, y); break;
+        case 16: launch_pat_r<C, 16>(st, V, s, sms, x, y); break;
+        case 32: launch_pat_r<C, 32>(st, V, s, sms, x, y); break;
+        default: launch_pat_plain<C, 0>(st, V, s, nrhs, x, y); break;
     }
 }
 
@@ -492,11 +625,11 @@ fe_status fe_spmv(fe_ctx* ctx, const fe_system* s, int32_t precision, int32_t nr
     const int64_t pat_blocks = ((int64_t)m->n_act + s->n_expl) * 3 * nrhs / 256 + 2;
     if (s->n_pat && terms && pat_blocks < (1ll << 31)) {
         if (precision == FE_PREC_FP64)
-            launch_spmv_pat<double2>(st, s, terms, nrhs, (const double2*)x, (double2*)y);
+            launch_spmv_pat<double2>(st, s, ctx->num_sms, terms, nrhs, (const double2*)x, (double2*)y);
         else if (precision == FE_PREC_MIXED)
-            launch_spmv_pat<float2>(st, s, terms, nrhs, (const float2*)x, (float2*)y);
+            launch_spmv_pat<float2>(st, s, ctx->num_sms, terms, nrhs, (const float2*)x, (float2*)y);
         else
-            launch_spmv_pat<float4>(st, s, terms, nrhs, (const float4*)x, (float4*)y);
+            launch_spmv_pat<float4>(st, s, ctx->num_sms, terms, nrhs, (const float4*)x, (float4*)y);
     } else if (precision == FE_PREC_FP64) {
         if (pow2 && nrhs >= 8)
             launch_spmm_rows<double2>(nrhs, st, ctx->num_sms, (const double2*)s->val64.ptr, s->stride, col, rp,
