@@ -110,6 +110,25 @@ __global__ void k_scan_sums(int* sums, int n_tiles, int* d_total) {
     if (threadIdx.x == 0) *d_total = carry;
 }
 
+// The last two passes in one for up to kScanFused tiles: every block adds the
+// sums of the tiles before its own (a few lines that stay in L2).
+constexpr int kScanFused = 2048;
+__global__ void __launch_bounds__(kScanThreads) k_scan_add(int* __restrict__ out, const int* __restrict__ tile_sums,
+                                                           int n_tiles, int64_t n, int* d_total) {
+    __shared__ int s_warp[32];
+    int before = 0, all = 0;
+    const bool last = (int)blockIdx.x == n_tiles - 1;
+    for (int t = threadIdx.x; t < (int)blockIdx.x; t += kScanThreads) before += tile_sums[t];
+    block_exclusive_scan(before, &all, s_warp);
+    if (last && threadIdx.x == 0) *d_total = all + tile_sums[blockIdx.x];
+    const int64_t base = (int64_t)blockIdx.x * kScanTile;
+#pragma unroll
+    for (int i = 0; i < kScanItems; ++i) {
+        const int64_t k = base + i * kScanThreads + threadIdx.x;
+        if (k < n) out[k] += all;
+    }
+}
+
 __global__ void k_scan_fix(int* __restrict__ out, const int* __restrict__ tile_sums, int64_t n) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) out[i] += tile_sums[i / kScanTile];
@@ -125,6 +144,11 @@ fe_status scan_exclusive(cudaStream_t st, const int* in, int* out, int64_t n, in
     int* sums = (int*)tmp.ptr;
     k_scan_tiles<<<(unsigned)tiles, kScanThreads, 0, st>>>(in, out, sums, n);
     FE_LAUNCHED();
+    if (tiles <= kScanFused) {
+        k_scan_add<<<(unsigned)tiles, kScanThreads, 0, st>>>(out, sums, (int)tiles, n, d_total);
+        FE_LAUNCHED();
+        return FE_OK;
+    }
     k_scan_sums<<<1, 1024, 0, st>>>(sums, (int)tiles, d_total);
     FE_LAUNCHED();
     k_scan_fix<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(out, sums, n);

@@ -118,7 +118,7 @@ __device__ double pen_entry(const TableParams& P, int f, int a, int al, int b, i
 // orientation f; n_mat + 6 + f the PEC-face table.
 __global__ void k_tables(TableParams P, double2* __restrict__ tab) {
     const int t = blockIdx.x;
-    const int idx = threadIdx.x;  // 0..575, block-major
+    const int idx = blockIdx.y * blockDim.x + threadIdx.x;  // 0..575, block-major
     const int blk = idx / 9, w = idx % 9;
     const int a = blk >> 3, b = blk & 7, al = w / 3, be = w % 3;
     Cx v = cx(0, 0);
@@ -173,6 +173,27 @@ __global__ void __launch_bounds__(256) k_assemble(const uint8_t* __restrict__ ma
     const unsigned az = dz < 0 ? 0x0Fu : dz > 0 ? 0xF0u : 0xFFu;
     const unsigned shared = lane < 27 ? (emask & ax & ay & az) : 0u;
     const unsigned exists = __ballot_sync(0xffffffffu, shared != 0);
+    // the 6 faces of the 8 elements, one or two per lane: on an absorbing face
+    // of the box, or against a PEC element (bit 6 p + f, in two words of 32)
+    unsigned ext[2], pec[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int t = 32 * h + lane, p = t / 6, f = t - 6 * p;
+        bool is_ext = false, is_pec = false;
+        if (t < 48 && ((emask >> p) & 1u)) {
+            const int ec[3] = {i - 1 + (p & 1), j - 1 + ((p >> 1) & 1), k - 1 + (p >> 2)}, dim[3] = {nx, ny, nz};
+            const int axis = f >> 1, side = f & 1;
+            if (side ? ec[axis] == dim[axis] - 1 : ec[axis] == 0) {
+                is_ext = (abc >> f) & 1u;  // symmetry-plane faces carry no surface term
+            } else {
+                int nb[3] = {ec[0], ec[1], ec[2]};
+                nb[axis] += side ? 1 : -1;
+                is_pec = mat[nb[0] + (int64_t)nx * (nb[1] + (int64_t)ny * nb[2])] == kPEC;
+            }
+        }
+        ext[h] = __ballot_sync(0xffffffffu, is_ext);
+        pec[h] = __ballot_sync(0xffffffffu, is_pec);
+    }
     if (!shared) return;
     const int slot = row_ptr[warp] + __popc(exists & ((1u << lane) - 1u));
 
@@ -198,20 +219,11 @@ __global__ void __launch_bounds__(256) k_assemble(const uint8_t* __restrict__ ma
             acc[q].y += v.y;
         }
         // faces of this element on the outer box or against a PEC element
-        const int ec[3] = {ei, ej, ek};
-        const int dim[3] = {nx, ny, nz};
 #pragma unroll
         for (int f = 0; f < 6; ++f) {
-            const int axis = f >> 1, side = f & 1;
-            const bool on_box = side ? ec[axis] == dim[axis] - 1 : ec[axis] == 0;
-            int tsel = -1;
-            if (on_box) {
-                if ((abc >> f) & 1u) tsel = n_mat + f;  // symmetry-plane faces carry no surface term
-            } else {
-                int nb[3] = {ei, ej, ek};
-                nb[axis] += side ? 1 : -1;
-                if (mat[nb[0] + (int64_t)nx * (nb[1] + (int64_t)ny * nb[2])] == kPEC) tsel = n_mat + 6 + f;
-            }
+            const int bit = 6 * p + f;
+            const bool on_ext = (ext[bit >> 5] >> (bit & 31)) & 1u, on_pec = (pec[bit >> 5] >> (bit & 31)) & 1u;
+            const int tsel = on_ext ? n_mat + f : (on_pec ? n_mat + 6 + f : -1);
             if (tsel >= 0) {
                 const double2* fv = tab + (size_t)tsel * 576 + (a * 8 + b) * 9;
 #pragma unroll
@@ -296,18 +308,22 @@ __global__ void k_row_class(const uint8_t* __restrict__ mat, int nx, int ny, int
     int c = -1;
     if (i >= 2 && i <= nx - 2 && j >= 2 && j <= ny - 2 && k >= 2 && k <= nz - 2) {
         // the 8 elements and their face neighbours lie inside the box
-        const int m = mat[(i - 1) + (int64_t)nx * ((j - 1) + (int64_t)ny * (k - 1))];
-        bool ok = m != kPEC && m < kMaxClasses;
-        for (int ez = 0; ez < 2 && ok; ++ez)
-            for (int ey = 0; ey < 2 && ok; ++ey)
-                for (int ex = 0; ex < 2 && ok; ++ex) {
-                    const int a = i - 1 + ex, b = j - 1 + ey, cc = k - 1 + ez;
-                    if (mat[a + (int64_t)nx * (b + (int64_t)ny * cc)] != m) ok = false;
-                    const int nb[6][3] = {{a - 1, b, cc}, {a + 1, b, cc}, {a, b - 1, cc},
-                                          {a, b + 1, cc}, {a, b, cc - 1}, {a, b, cc + 1}};
-                    for (int f = 0; f < 6 && ok; ++f)
-                        if (mat[nb[f][0] + (int64_t)nx * (nb[f][1] + (int64_t)ny * nb[f][2])] == kPEC) ok = false;
-                }
+        const int sx = nx, sz = nx * ny;  // at most 2^24 elements
+        const uint8_t* e = mat + (i - 1) + sx * (j - 1) + sz * (k - 1);
+        const int m = e[0];
+        bool ok = m != kPEC && m < kMaxClasses && e[1] == m && e[sx] == m && e[sx + 1] == m && e[sz] == m &&
+                  e[sz + 1] == m && e[sz + sx] == m && e[sz + sx + 1] == m;
+        if (ok) {
+            bool pec = false;  // no short cut: the 24 loads are in flight together
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int a = u & 1, b = u >> 1;
+                const uint8_t *x = e + sx * a + sz * b, *y = e + a + sz * b, *z = e + a + sx * b;
+                pec |= (x[-1] == kPEC) | (x[2] == kPEC) | (y[-sx] == kPEC) | (y[2 * sx] == kPEC) | (z[-sz] == kPEC) |
+                       (z[2 * sz] == kPEC);
+            }
+            ok = !pec;
+        }
         // E: no neighbour on a conductor surface either (its held columns would
         // differ from the class stencil): no PEC in the 4 x 4 x 4 elements around
         for (int ez = -2; ez < 2 && ok && form_e; ++ez)
@@ -317,7 +333,11 @@ __global__ void k_row_class(const uint8_t* __restrict__ mat, int nx, int ny, int
         if (ok) c = m;
     }
     cls[r] = (signed char)c;
-    if (c >= 0) atomicMin(&rep[c], r);
+    // one update per class and warp (most rows of a mesh are of one class)
+    if (c >= 0) {
+        const unsigned same = __match_any_sync(__activemask(), c);
+        if ((int)(threadIdx.x & 31) == __ffs(same) - 1 && *(volatile int*)&rep[c] > r) atomicMin(&rep[c], r);
+    }
 }
 
 // One warp per class: copies the 27 blocks of the class's first regular row
@@ -496,7 +516,8 @@ fe_status fe_assemble(fe_ctx* ctx, const fe_mesh* m, double freq_hz, int32_t pre
     }
     int* d_status = (int*)ctx->small.ptr + 8;
     cudaMemsetAsync(d_status, 0, sizeof(int), st);
-    k_tables<<<n_tab, 576, 0, st>>>(P, (double2*)s->tables.ptr);
+    // small blocks: the FP64 work of a table spreads over nine SMs
+    k_tables<<<dim3(n_tab, 9), 64, 0, st>>>(P, (double2*)s->tables.ptr);
     {
         count_launches(1);
         cudaError_t ce = cudaGetLastError();
@@ -516,7 +537,9 @@ fe_status fe_assemble(fe_ctx* ctx, const fe_mesh* m, double freq_hz, int32_t pre
         return fail(e);
     };
     if ((e = group_rows(ctx, s, row_group, d_flags)) != FE_OK) return fail_group(e);
-    const int threads = 256;
+    // one warp per block for the few first rows, so that each has an SM's FP64
+    // pipe to itself (80 rows: 48 us in blocks of eight warps)
+    const int threads = s->n_pat ? 32 : 256;
     const int n_asm = s->n_pat ? s->n_pat : m->n_act;
     const unsigned blocks = (unsigned)(((int64_t)n_asm * 32 + threads - 1) / threads);
     k_assemble<<<blocks, threads, 0, st>>>((const uint8_t*)m->material.ptr, m->nx, m->ny, m->nz, m->n_mat,
