@@ -452,7 +452,8 @@ typedef struct fe_serve_opts {
     int32_t max_job_ctas;  /* CTAs one request may take (a cap leaves room for requests that arrive while a
                               large one runs); 0: three quarters of max_ctas; max_ctas: no cap */
     int32_t seg_iters;     /* Krylov iterations per segment; 0 (default): each request runs as many as fill
-                              about 25 ms at its own measured time per iteration (64 in its first segment) */
+                              about 25 ms at its own measured time per iteration (its first segment: 64 when it
+                              runs alone, else an estimate from its size) */
     int32_t recurrence;    /* fe_recurrence of every request's solve; default FE_RECURRENCE_EXPANDED (a stream of
                               voxel cubes at 1-6 GHz, 8-50 nodes per side: 4.13 solves/s and all of the first 128
                               requests converged, against 2.24 and 127 with FE_RECURRENCE_CG) */

@@ -77,13 +77,31 @@ struct ServeReq {
 // Segments last about kSegTargetMs: each request runs as many iterations as
 // its own measured time per iteration allows, so that a small request
 // launched beside a large one keeps its SMs busy for the whole segment.
+// Before the first measurement a request that runs beside others takes an
+// estimate from its size: 64 iterations, as it once ran, end after a few
+// milliseconds and its SMs then wait for the requests beside it (a burst of 12
+// small requests spent 25 of its 70 ms so).  A request alone does start with
+// 64, so that others that arrive with it join it soon.
 constexpr double kSegTargetMs = 25.0;
 constexpr int kSegFirst = 64;
 
-int segment_iters(const fe_serve_opts& o, const ServeReq* q) {
+// Milliseconds per iteration of a request on n_cta CTAs: barriers and
+// latencies, and the CTA's work items (unknowns x columns) at the rate measured
+// on wide tiles; systems without row patterns take about four times as long.
+double guess_ms_per_iter(const ServeReq* q, int prec, int width, int n_cta) {
+    const double items = (double)q->n_dof * width / n_cta;
+    const double ns = prec == FE_PREC_FP64 ? 35.0 : (prec == FE_PREC_MIXED ? 22.0 : 12.0);
+    return 0.015 + items * ns * (q->sys && q->sys->n_pat ? 1.0 : 4.0) * 1e-6;
+}
+
+int segment_iters(const fe_serve_opts& o, const ServeReq* q, bool alone, int width, int n_cta) {
     if (o.seg_iters > 0) return o.seg_iters;
-    if (!(q->ms_per_iter > 0.0)) return kSegFirst;
-    return (int)std::max(16.0, std::min(1e6, kSegTargetMs / q->ms_per_iter));
+    double ms = q->ms_per_iter;
+    if (!(ms > 0.0)) {
+        if (alone) return kSegFirst;
+        ms = guess_ms_per_iter(q, o.precision, width, n_cta);
+    }
+    return (int)std::max(16.0, std::min(1e6, kSegTargetMs / ms));
 }
 
 int width_slot(int width) {
@@ -255,12 +273,13 @@ bool worker_turn(fe_server* S) {
     std::vector<int> ctas[6], iters[6];
     std::vector<ServeReq*> in_seg[6];
     int n_seg = 0;
+    const bool alone = n == 1;
     for (int i = 0; i < n; ++i) {
         if (n_cta[i] <= 0) continue;
         const int k = width_slot(width[i]);
         jobs[k].push_back(S->ready[i]->job);
         ctas[k].push_back(n_cta[i]);
-        iters[k].push_back(segment_iters(S->o, S->ready[i]));
+        iters[k].push_back(segment_iters(S->o, S->ready[i], alone, width[i], n_cta[i]));
         in_seg[k].push_back(S->ready[i]);
         ++n_seg;
     }
