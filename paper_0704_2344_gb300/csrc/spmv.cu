@@ -369,6 +369,12 @@ static void launch_spmv_warp(int R, unsigned blocks, cudaStream_t st, const C* v
 //           consecutive rows per thread, which share two of every three
 //           entries along a grid line.  Walking a range keeps a row's lines in
 //           L1 for the rows above and beside it.
+//
+// Measured per product, from the stored blocks and here (in brackets: all by
+// the plain form): FP32 pairs, 9 261 rows 10.1 and 4.9 us (9.1); complex64,
+// 80^3 aircraft 196 and 28.9 us (32.4), 60^3 aircraft with 16 columns 306 and
+// 128 us (149); complex128, 48^3 nodes with 3 columns 840 and 106 us, 0.8 of
+// the FP64 pipe's rate on the non-zero terms.
 // ---------------------------------------------------------------------------
 template <typename C, int R_>
 __device__ __forceinline__ void pat_item(const PatView<C>& V, const C* __restrict__ x, C* __restrict__ y, int row,
@@ -599,6 +605,23 @@ static void launch_spmv_pat(cudaStream_t st, const fe_system* s, int sms, const 
     }
 }
 
+// Products so small that neither the lanes nor the bandwidth bound them: the
+// patterns' chain of dependent loads (row, table, line, term, entry) is one
+// longer than the stored blocks', which stay in L2.  Measured per call:
+// complex64, 1 column, 9 261 rows 8.2 us by patterns and 6.2 stored, equal at
+// 15 625 rows; 2 columns, 5 832 rows 8.2 and 6.2; 4 columns and more, patterns
+// are ahead from the start, but for 8 and 16 between the range where two lanes
+// share an item and the one that fills the lanes (8 columns, 9 261 rows 14.4 and
+// 12.3; 5 832 rows 10.4 and 12.3, 15 625 rows 14.4 and 18.5).  FP32 pairs,
+// 2 197 rows: 1 column 8.2 and 6.2, 4 columns 10.3 and 9.2; equal at 4 096 rows.
+// FP64 is ahead at every size.
+static bool small_stored(int precision, int n_rows, int nrhs) {
+    const int64_t items = (int64_t)n_rows * 3 * nrhs;
+    if (precision == FE_PREC_MIXED)
+        return nrhs <= 2 ? n_rows <= 9300 : (nrhs == 8 || nrhs == 16) && items > kSplitItems && items <= 240000;
+    return precision == FE_PREC_DF && (nrhs <= 2 || nrhs == 4) && n_rows <= 2200;
+}
+
 }  // namespace fe
 
 using namespace fe;
@@ -623,7 +646,7 @@ fe_status fe_spmv(fe_ctx* ctx, const fe_system* s, int32_t precision, int32_t nr
                         : precision == FE_PREC_MIXED ? s->pat_t32.ptr
                         : precision == FE_PREC_DF ? s->pat_tdf.ptr : nullptr;
     const int64_t pat_blocks = ((int64_t)m->n_act + s->n_expl) * 3 * nrhs / 256 + 2;
-    if (s->n_pat && terms && pat_blocks < (1ll << 31)) {
+    if (s->n_pat && terms && pat_blocks < (1ll << 31) && !small_stored(precision, m->n_act, nrhs)) {
         if (precision == FE_PREC_FP64)
             launch_spmv_pat<double2>(st, s, ctx->num_sms, terms, nrhs, (const double2*)x, (double2*)y);
         else if (precision == FE_PREC_MIXED)

@@ -28,7 +28,7 @@ def _random_materials(n=9, kinds=6, seed=11):
 
 
 def _lossy_slab():
-    prob = W.pec_box_problem(12, 3e9, np.random.default_rng(4))
+    prob = W.pec_box_problem(13, 3e9, np.random.default_rng(4))
     prob.material[2:4, 2:9, 3:11][prob.material[2:4, 2:9, 3:11] != W.PEC] = 1
     prob.eps_r = np.array([1.0, 2.5 - 0.4j])
     prob.mu_r = np.array([1.0, 1.2 - 0.1j])
@@ -100,6 +100,40 @@ def test_solve_matches_the_oracle(fe, ctx, name, precision, nrhs):
             _, x, rep = fe.fe_solve_batch(ctx, s, waves, maps.n_dof, fe.solve_opts(precision=prec, recurrence=rec))
             assert all(r["status"] == 0 for r in rep)
             assert fem.true_relative_residual(A, x, B).max() <= 1e-8
+    finally:
+        fe.fe_system_destroy(s)
+        fe.fe_mesh_destroy(m)
+
+
+@pytest.fixture(scope="module")
+def walk_case():
+    """31 x 34 x 30 nodes with a PEC block and a lossy slab: enough rows for the walks from 4 columns on."""
+    prob = W.empty_box((30, 33, 29))
+    prob.material[10:17, 12:19, 8:15] = W.PEC
+    prob.material[3:6, 4:30, 5:20] = 1
+    prob.eps_r = np.array([1.0, 2.5 - 0.4j])
+    prob.mu_r = np.array([1.0, 1.2 - 0.1j])
+    maps = fem.mesh_maps(prob)
+    return prob, maps, fem.assemble(prob, maps=maps)
+
+
+@pytest.mark.parametrize("nrhs", [1, 2, 4, 8, 32])
+def test_walk_product_matches_the_oracle(fe, ctx, walk_case, nrhs):
+    import torch
+
+    prob, maps, A = walk_case
+    rng = np.random.default_rng(nrhs)
+    x = (rng.standard_normal((maps.n_dof, nrhs)) + 1j * rng.standard_normal((maps.n_dof, nrhs))).astype(np.complex64)
+    m = fe.fe_mesh_create_from(ctx, prob)
+    s = fe.fe_assemble(ctx, m, prob.freq_hz, fe.FE_PREC_MIXED)
+    try:
+        xd = torch.from_numpy(x).cuda()
+        yd = torch.empty_like(xd)
+        torch.cuda.synchronize()
+        fe.fe_spmv(ctx, s, fe.FE_PREC_MIXED, nrhs, xd, yd)
+        fe.fe_ctx_synchronize(ctx)
+        err = np.abs(yd.cpu().numpy() - A @ x.astype(complex))
+        assert np.all(err <= 5e-6 * (abs(A) @ np.abs(x)) + 1e-300)
     finally:
         fe.fe_system_destroy(s)
         fe.fe_mesh_destroy(m)
