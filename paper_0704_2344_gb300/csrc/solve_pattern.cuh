@@ -15,6 +15,13 @@
 //   - 512 threads with 128 registers instead of 1024 with 64: a CTA of a
 //     mid-sized system has some 600 items, so the phases are bound by latency,
 //     and registers for loads in flight count more than warps.
+//
+// Bound by latency: of the 16.5 us an iteration of the 3-wavelength cube takes
+// with FP32 pairs, the two grid barriers take 4.3 and the rest is short phases
+// of dependent operations; FP64 keeps its pipe about half busy.  Measured, us
+// per iteration, solve_kernels.cuh and here: FP32 pairs 10^3 20.1 and 10.7, 30^3
+// 25.6 and 16.5, 40^3 expanded 90 and 26.7, 18^3 with 12 columns 106 and 36;
+// FP64 20^3 48 and 19.6; complex64 20^3 14.6 (17.4 before its sums were paired).
 #pragma once
 
 #include "solve_kernels.cuh"
@@ -113,14 +120,49 @@ __device__ __noinline__ bool pat_reduce(const SolveParams& P, int cta, const dou
     return true;
 }
 
+// Warp sums of N doubles over the lanes of one column (lane % R), two values to
+// a butterfly step while there are two: a lane hands one of them over and keeps
+// the other.  Five values take 8 additions a lane instead of 25; an FP64
+// addition holds an SM's FP64 pipe for 16 cycles a warp, so that the 25 of 16
+// warps took 3 us of an iteration.  (FP32 pairs, on wider pipes, keep one value
+// to a step: 1 us.)  Afterwards a lane's w[k] is the sum of value
+// (k << shift) | value, the same in the lanes that differ only in bits `same`.
+struct WarpSums {
+    int value = 0, same = 0, left = 0, shift = 0;
+};
+__device__ __forceinline__ double sum_from(double keep, double give, int o) {
+    return keep + __shfl_xor_sync(0xffffffffu, give, o);
+}
+template <int O, int R, int N>
+__device__ __forceinline__ void warp_sums(double* w, int lane, WarpSums& m) {
+    if constexpr (O < R) {
+        m.left = N;
+    } else if constexpr (N == 1) {
+        w[0] = sum_from(w[0], w[0], O);
+        m.same |= O;
+        warp_sums<O / 2, R, 1>(w, lane, m);
+    } else {
+        const bool up = lane & O;
+#pragma unroll
+        for (int k = 0; k < N / 2; ++k) {
+            const double a = w[2 * k], b = w[2 * k + 1];
+            w[k] = sum_from(up ? b : a, up ? a : b, O);
+        }
+        if constexpr (N % 2) w[N / 2] = sum_from(w[N - 1], w[N - 1], O);  // the odd one out; used where !up
+        if (up) m.value |= 1 << m.shift;
+        ++m.shift;
+        warp_sums<O / 2, R, (N + 1) / 2>(w, lane, m);
+    }
+}
+
 // Sum over the CTA of per-thread values, per column (thread t holds column
 // t % R): NV of them, FP32 pairs (f[2k] + f[2k + 1]) or doubles.
 template <int R, int NV, bool kPair>
 __device__ __forceinline__ void pat_colsum(const float* f, const double* d, double* s_red, double* s_in) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if constexpr (kPair) {
 #pragma unroll
-    for (int k = 0; k < NV; ++k) {
-        if (kPair) {
+        for (int k = 0; k < NV; ++k) {
             float h = f[2 * k], l = f[2 * k + 1];
 #pragma unroll
             for (int o = 16; o >= R; o >>= 1) {
@@ -128,11 +170,17 @@ __device__ __forceinline__ void pat_colsum(const float* f, const double* d, doub
                 df_add(h, l, h2, l2);
             }
             if (lane < R) ((float2*)s_red)[(k * kPW + warp) * R + lane] = make_float2(h, l);
-        } else {
-            double w = d[k];
+        }
+    } else {
+        double w[NV];
 #pragma unroll
-            for (int o = 16; o >= R; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
-            if (lane < R) s_red[(k * kPW + warp) * R + lane] = w;
+        for (int k = 0; k < NV; ++k) w[k] = d[k];
+        WarpSums m;
+        warp_sums<16, R, NV>(w, lane, m);
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+            const int v = (k << m.shift) | m.value;
+            if (k < m.left && v < NV && !(lane & m.same)) s_red[(v * kPW + warp) * R + lane % R] = w[k];
         }
     }
     __syncthreads();
