@@ -435,7 +435,7 @@ def run_ours(args, rank, world, local_rank, precision_name):
                 "alu_view": {"method_tflops": round(method_flops / launch_s / 1e12, 3) if launch_s > 0 else None,
                              "fp32_peak_tflops": round(FP32_PEAK_TFLOPS, 2)}}
     roof.update(work)
-    roof["stencil_reduced_bytes_per_launch"] = int(alg / steps)   # what the class-stencil product actually reads
+    roof["stencil_reduced_bytes_per_launch"] = int(alg / steps)   # what products from per-material stencils read
     roof.update(common)
     roof["traffic"] = recorded_traffic(args.workload, precision_name)   # ncu DRAM bytes per launch (or None)
     roof["launch_ms"] = round(launch_ms, 4)

@@ -195,16 +195,19 @@ fe_status fe_assemble(fe_ctx* ctx, const fe_mesh* m, double freq_hz, int32_t pre
  * else FE_ERR_INVALID_ARG), dinv_c128[n_nodes*9*2 doubles]. */
 fe_status fe_system_export(fe_ctx* ctx, const fe_system* s, void* vals_c128, void* vals_c64, void* dinv_c128);
 /* Block dictionary (complex64 and FP32-pair systems): equal local
- * configurations of the voxel mesh give bitwise equal 3x3 blocks, so the
- * system also keeps each distinct block once (at most 4096 of them) with an
- * index per stored block; single-column solves read explicit rows through it
- * when it fits in shared memory.  dict_blocks counts the distinct blocks, 0
- * when there are too many (the products then read the stored values).
+ * configurations of the voxel mesh give bitwise equal 3x3 blocks.  Whole rows
+ * repeat too: the system keeps the non-zero entries of each distinct block row
+ * once (a row pattern), and products and solves read those.  A mesh with too
+ * many distinct rows (above an eighth of its nodes, at least 128 and at most
+ * 2048) has no patterns; it keeps each distinct block once (at most 4096)
+ * with an index per stored block, and its products read those or the stored
+ * values.  dict_blocks counts the distinct blocks either way, 0 when there
+ * are too many.
  *
  * Regular rows (interior nodes whose eight elements are active, of one
  * material, with no outer or PEC face) all carry the same 27 blocks per
- * material; the Krylov products read them from a per-material stencil instead
- * of the stored blocks.  The counts say how many rows take each path. */
+ * material; without patterns the Krylov products read them from a
+ * per-material stencil.  The counts say how many rows are of each kind. */
 typedef struct fe_system_stats {
     int32_t precision;         /* as assembled */
     int32_t dict_blocks;       /* distinct 3x3 blocks in the block dictionary (0: none) */
@@ -311,8 +314,8 @@ fe_status fe_spmv_half(fe_ctx* ctx, const fe_system* s, int32_t precision, int32
  * runs the autotuner: short trial launches (32 iterations of the first
  * columns) for every tile width in {8, 16, 32} up to the column count and
  * grids of all or three quarters of the SMs, timed with CUDA events; the
- * fastest per column and iteration is kept for that shape in a process-wide
- * cache and reported in fe_solve_stats.  Fewer right-hand sides use the
+ * widest tile within 5 % of the least device time for one iteration of all
+ * columns is kept for that shape in a process-wide cache and reported in fe_solve_stats.  Fewer right-hand sides use the
  * widest power of two up to their count.
  * ---------------------------------------------------------------------- */
 /* The form of the COCG step length alpha = gamma / (p^T A p).  Every
@@ -402,10 +405,11 @@ fe_status fe_solve_rhs(fe_ctx* ctx, const fe_system* s, int32_t nrhs, const void
  * optional host array of nrhs reports.
  *
  * Scratch: the call keeps all of its workspace in one file-scope device array
- * of 32 MiB (every GPU that loads the library holds it until the process
+ * of 34 MiB (every GPU that loads the library holds it until the process
  * exits); it calls no cudaMalloc / cudaFree and no allocating routine.  The
  * need is 80 bytes per unknown and right-hand side in the FP64 and FP32-pair
- * modes and 88 in the mixed mode, plus a few KiB, so n_dof * nrhs may reach
+ * modes and 88 in the mixed mode, plus a few KiB, within 32 MiB (the rest
+ * holds partial sums), so n_dof * nrhs may reach
  * about 415 000 (FP64, FP32 pairs) or 380 000 (mixed); a larger problem is
  * rejected with FE_ERR_INVALID_ARG and a message naming the bytes it would
  * need.  The first call on a device looks the array's device address up

@@ -11,9 +11,10 @@
 // mode, complex128 in the plain mode), the FP64 solution update, and every
 // convergence decision.  CTAs own contiguous ranges of block rows and meet
 // at a grid barrier whose wait is bounded in time; the barrier also performs
-// the dot-product reductions: each CTA publishes its partial sums and the
-// last CTA to arrive adds them in a fixed order, so every CTA sees bitwise the
-// same scalars and takes the same branch.
+// the dot-product reductions: each CTA publishes its partial sums and every
+// CTA adds all of them in one fixed order, so every CTA sees bitwise the same
+// scalars and takes the same branch.  Systems with row patterns and block
+// Jacobi run solve_pattern.cuh's kernels, the others solve_kernels.cuh's.
 #include "krylov.cuh"
 
 #include <algorithm>
