@@ -235,7 +235,7 @@ def kernel_hash() -> str:
     import hashlib
     csrc = ROOT / "paper_0704_2344_gb300" / "csrc"
     h = hashlib.sha256()
-    for f in ("solve.cu", "solve_kernels.cuh", "krylov.cuh", "fe_internal.cuh"):
+    for f in ("solve.cu", "solve_kernels.cuh", "solve_pattern.cuh", "patterns.cuh", "krylov.cuh", "fe_internal.cuh"):
         h.update((csrc / f).read_bytes())
     return h.hexdigest()[:16]
 
@@ -415,7 +415,7 @@ def run_ours(args, rank, world, local_rank, precision_name):
         # complex128 products run on the FP64 pipes (1/64 of the FP32 rate):
         # 8 flops per complex multiply-add against that rate
         achieved = method_flops / launch_s / 1e12 if launch_s > 0 else None
-        roof = {"kernel": f"k_solve<double,{tile_w}> (persistent COCG, FP64"
+        roof = {"kernel": f"{'k_solve' if bicp else 'k_solve_pat'}<double,{tile_w}> (persistent COCG, FP64"
                           + (", block incomplete Cholesky)" if bicp else ")"), "bound": "alu",
                 "achieved": round(achieved, 4) if achieved else None, "peak": round(FP64_PEAK_TFLOPS, 3),
                 "unit": "TFLOP/s", "frac": round(achieved / FP64_PEAK_TFLOPS, 4) if achieved else None,
@@ -425,13 +425,14 @@ def run_ours(args, rank, world, local_rank, precision_name):
                              "frac": round(method_bytes / launch_s / 1e9 / hbm_peak, 4)} if launch_s > 0 else None}
     else:
         achieved = method_bytes / launch_s / 1e9 if launch_s > 0 else None
-        roof = {"kernel": f"k_solve<{'DFloat' if base == 'df' else 'float'},{tile_w}> (persistent COCG, "
+        roof = {"kernel": f"k_solve_pat<{'DFloat' if base == 'df' else 'float'},{tile_w}> (persistent COCG, "
                           + ("FP32-pair" if base == "df" else "complex64") + " products)", "bound": "hbm",
                 "achieved": round(achieved, 1) if achieved else None, "peak": hbm_peak, "unit": "GB/s",
                 "frac": round(achieved / hbm_peak, 4) if achieved else None,
                 "peak_source": f"{hbm_src} (MEASURED_PEAKS.json hbm_gbs)" if hbm_src == "measured" else hbm_src,
                 "work": "(products_per_launch * bytes_per_product + fp64_products_per_launch * "
                         "bytes_per_fp64_product) / (launch_ms * 1e-3) / 1e9",
+                "note": "the method's bytes; products from row patterns do not read the stored blocks",
                 "alu_view": {"method_tflops": round(method_flops / launch_s / 1e12, 3) if launch_s > 0 else None,
                              "fp32_peak_tflops": round(FP32_PEAK_TFLOPS, 2)}}
     roof.update(work)
