@@ -137,13 +137,6 @@ __device__ __forceinline__ void put_term(float4* p, double v, int code) {
     *p = make_float4(h, __double2float_rn(v - (double)h), __int_as_float(code), 0.f);
 }
 
-// Cost of a row in a product, in terms: its steps and the fixed work of a
-// component (line lookup, five inner products, the store), about eight terms;
-// the interior's steps skip the term codes.
-__host__ __device__ __forceinline__ int pattern_cost(int n_re, int n_im, bool diag) {
-    return diag ? 30 : n_re + n_im + 8;
-}
-
 // Term lists of one pattern per block, one warp per component: lane k < nb
 // holds the component's three entries of block k.  Parts below 2^-52 of the
 // row's largest are sums that cancel and count as zero.
@@ -151,7 +144,7 @@ __global__ void __launch_bounds__(96) k_pat_terms(const int* __restrict__ first_
                                                   const int* __restrict__ col, const int* __restrict__ node_id,
                                                   const double2* __restrict__ val, int64_t stride, int sy, int sz,
                                                   int4* __restrict__ tab, double2* __restrict__ t64,
-                                                  float2* __restrict__ t32, float4* __restrict__ tdf,
+                                                  float2* __restrict__ t32, float4* __restrict__ tdf, int cost_shift,
                                                   int* __restrict__ flags) {
     __shared__ int s_nre[3], s_nim[3], s_diag[3];
     const int p = blockIdx.x, al = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -249,7 +242,7 @@ __global__ void __launch_bounds__(96) k_pat_terms(const int* __restrict__ first_
     }
     if (threadIdx.x == 0) {
         tab[p] = make_int4(p * kPatStride, n_re, n_im, diag ? 1 : 0);
-        const int cost = pattern_cost(n_re, n_im, diag);
+        const int cost = scaled_cost(row_cost(n_re, n_im, diag), cost_shift);
         atomicMin(flags + 3, cost);
         atomicMax(flags + 4, cost);
     }
@@ -288,7 +281,7 @@ __global__ void __launch_bounds__(256) k_pat_spread(const int* __restrict__ grou
                                                     double2* __restrict__ dinv64, float2* __restrict__ dinv32,
                                                     float4* __restrict__ dinvdf, const int* __restrict__ node_id,
                                                     uint16_t* __restrict__ pat_id, int4* __restrict__ pat_row,
-                                                    int* __restrict__ cost, int* __restrict__ expl) {
+                                                    int cost_shift, int* __restrict__ cost, int* __restrict__ expl) {
     const int r = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
     if (r >= n) return;
     const int id = __ldg(group + r);
@@ -310,7 +303,7 @@ __global__ void __launch_bounds__(256) k_pat_spread(const int* __restrict__ grou
         const int4 t = __ldg(tab + id);
         pat_id[r] = (uint16_t)id;
         pat_row[r] = make_int4(3 * t.x, t.y | t.z << 10 | t.w << 20, __ldg(node_id + r), id);
-        cost[r] = pattern_cost(t.y, t.z, t.w != 0);
+        cost[r] = scaled_cost(row_cost(t.y, t.z, t.w != 0), cost_shift);
         expl[r] = t.w ? 0 : 1;
     }
 }
@@ -399,6 +392,7 @@ fe_status build_patterns(fe_ctx* ctx, fe_system* s, const DevBuf& row_group, int
     if ((e = dev_alloc(st, s->pat_list, (size_t)n * sizeof(int))) != FE_OK) return done(e);
     if ((e = dev_alloc(st, expl, (size_t)n * sizeof(int))) != FE_OK) return done(e);
     const int sy = m->nx + 1, sz = (m->nx + 1) * (m->ny + 1);
+    const int shift = cost_shift(n);
     const int* rp = (const int*)m->row_ptr.ptr;
     const int* first = (const int*)s->pat_first.ptr;
     int* cost = (int*)s->pat_cost.ptr;
@@ -407,11 +401,12 @@ fe_status build_patterns(fe_ctx* ctx, fe_system* s, const DevBuf& row_group, int
     k_pat_terms<<<n_pat, 96, 0, st>>>(first, rp, (const int*)m->col_idx.ptr, (const int*)m->node_id.ptr,
                                       (const double2*)s->val64.ptr, s->stride, sy, sz, (int4*)s->pat_tab.ptr,
                                       (double2*)s->pat_t64.ptr, (float2*)s->pat_t32.ptr, (float4*)s->pat_tdf.ptr,
-                                      d_flags);
+                                      shift, d_flags);
     k_pat_spread<<<(unsigned)(((int64_t)n * 32 + 255) / 256), 256, 0, st>>>(
         (const int*)row_group.ptr, first, (const int4*)s->pat_tab.ptr, rp, s->stride, n, (double2*)s->val64.ptr,
         (float2*)s->val32.ptr, (float4*)s->valdf.ptr, (double2*)s->dinv64.ptr, (float2*)s->dinv32.ptr,
-        (float4*)s->dinvdf.ptr, (const int*)m->node_id.ptr, (uint16_t*)s->pat_id.ptr, (int4*)s->pat_row.ptr, cost, (int*)expl.ptr);
+        (float4*)s->dinvdf.ptr, (const int*)m->node_id.ptr, (uint16_t*)s->pat_id.ptr,
+        (int4*)s->pat_row.ptr, shift, cost, (int*)expl.ptr);
     count_launches(2);
     if ((e = scan_exclusive(st, cost, cost, n, d_totals, ctx->scan_tmp)) != FE_OK) return done(e);
     cudaMemcpyAsync(cost + n, d_totals, sizeof(int), cudaMemcpyDeviceToDevice, st);

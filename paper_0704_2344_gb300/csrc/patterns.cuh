@@ -24,6 +24,7 @@
 #pragma once
 
 #include "krylov.cuh"
+#include "row_cost.cuh"
 
 namespace fe {
 

@@ -1460,9 +1460,7 @@ void size_pat(SolveParams& P, int n_cta, size_t& dyn) {
     P.n_cta = n_cta;
     P.pat_half = (int64_t)n_cta * kPatNV * R;
     P.red_bytes = (int)(kPatNV * kPW * R * sizeof(double));
-    // a CTA's range costs at most total / n_cta plus one row
-    const int64_t bound = std::min<int64_t>(P.n_rows, (P.cost_total / n_cta + P.cost_max) / P.cost_min + 2);
-    const int64_t rows = (bound + 3) & ~3ll;
+    const int64_t rows = (cta_rows_bound(P.n_rows, P.cost_total, n_cta, P.cost_min, P.cost_max) + 3) & ~3ll;
     P.pat_rows_max = rows * kPatRowBytes <= kPatRowsBytes ? (int)rows : 0;
     P.pat_terms_max = kPatTermBytes / (int)sizeof(C);
     int64_t used = P.red_bytes + (((int64_t)P.pat_rows_max * kPatRowBytes + 15) & ~15ll) + kPatTermBytes +
