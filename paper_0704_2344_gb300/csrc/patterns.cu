@@ -138,8 +138,11 @@ __device__ __forceinline__ void put_term(float4* p, double v, int code) {
 }
 
 // Term lists of one pattern per block, one warp per component: lane k < nb
-// holds the component's three entries of block k.  Parts below 2^-52 of the
-// row's largest are sums that cancel and count as zero.
+// holds the component's three entries of block k.  A part is left out only
+// where the stored one is zero: the contributions of a uniform material that
+// cancel do so exactly (they are the same table entries with opposite signs),
+// and any other part is data however small it is beside the row's largest (a
+// loss tangent of 1e-17 alone makes the imaginary parts).  NaN is not zero.
 __global__ void __launch_bounds__(96) k_pat_terms(const int* __restrict__ first_of_id, const int* __restrict__ row_ptr,
                                                   const int* __restrict__ col, const int* __restrict__ node_id,
                                                   const double2* __restrict__ val, int64_t stride, int sy, int sz,
@@ -150,15 +153,10 @@ __global__ void __launch_bounds__(96) k_pat_terms(const int* __restrict__ first_
     const int p = blockIdx.x, al = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int row = first_of_id[p], s0 = row_ptr[row], nb = row_ptr[row + 1] - s0;
     double2 v[3];
-    double amax = 0.0;
     int line = 0, dx = 0;
 #pragma unroll
     for (int be = 0; be < 3; ++be) v[be] = make_double2(0.0, 0.0);
     if (lane < nb) {
-        for (int q = 0; q < 9; ++q) {
-            const double2 e = val[q * stride + s0 + lane];
-            amax = fmax(amax, fmax(fabs(e.x), fabs(e.y)));
-        }
 #pragma unroll
         for (int be = 0; be < 3; ++be) v[be] = val[(3 * al + be) * stride + s0 + lane];
         // grid offset of the column, split into (dx, dy, dz) by the extents
@@ -166,15 +164,12 @@ __global__ void __launch_bounds__(96) k_pat_terms(const int* __restrict__ first_
         dx = o % sy - id % sy;
         line = ((o / sy) % (sz / sy) - (id / sy) % (sz / sy) + 1) + 3 * (o / sz - id / sz + 1);
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) amax = fmax(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-    const double tiny = 2.220446049250313e-16 * amax;
     bool re[3], im[3], offdiag = false;
     int cre = 0, cim = 0;
 #pragma unroll
     for (int be = 0; be < 3; ++be) {
-        re[be] = fabs(v[be].x) > tiny;
-        im[be] = fabs(v[be].y) > tiny;
+        re[be] = !(v[be].x == 0.0);
+        im[be] = !(v[be].y == 0.0);
         cre += re[be];
         cim += im[be];
         offdiag = offdiag || im[be] || (be != al && re[be]);
