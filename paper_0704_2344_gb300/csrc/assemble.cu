@@ -576,13 +576,34 @@ fe_status fe_assemble(fe_ctx* ctx, const fe_mesh* m, double freq_hz, int32_t pre
         (const signed char*)s->row_class.ptr, (const StencilSet*)s->stencil.ptr, (const int*)m->row_ptr.ptr, m->n_act,
         d_counts);
     count_launches(3);
+    // Without patterns the products read the stored blocks, the class stencils
+    // and the block dictionary, and their rows are split by these costs, in
+    // units of one stored block of an explicit row: a general-stencil row
+    // costs 18 (complex64) or 27 (FP32 pairs, read through the block
+    // dictionary like an explicit row) such blocks, a diagonal-stencil row 10
+    // or 9 (per-CTA product times measured on GB300 and fitted to these three
+    // row kinds).  The third prefix counts the stored blocks of explicit rows
+    // only: a solve CTA packs its explicit rows' values at 9 times that prefix.
+    const int weights[3][3] = {{1, 18, 10}, {1, 27, 9}, {1, 0, 0}};
+    DevBuf* bufs[3] = {&s->cost_prefix, &s->cost_prefix_alu, &s->expl_prefix};
+    int* d_total = (int*)ctx->small.ptr + 24;
+    for (int k = 0; k < 3 && !s->n_pat; ++k) {
+        if ((e = dev_alloc(st, *bufs[k], (size_t)(m->n_act + 1) * sizeof(int))) != FE_OK) return fail(e);
+        int* cp = (int*)bufs[k]->ptr;
+        k_row_cost<<<(unsigned)((m->n_act + 255) / 256), 256, 0, st>>>(
+            (const signed char*)s->row_class.ptr, (const StencilSet*)s->stencil.ptr, (const int*)m->row_ptr.ptr,
+            m->n_act, weights[k][0], weights[k][1], weights[k][2], cp);
+        count_launches(1);
+        if ((e = scan_exclusive(st, cp, cp, m->n_act, d_total + k, ctx->scan_tmp)) != FE_OK) return fail(e);
+        cudaMemcpyAsync(cp + m->n_act, d_total + k, sizeof(int), cudaMemcpyDeviceToDevice, st);
+    }
     int* h = ctx->h_small;
     if (s->n_pat && precision != FE_PREC_FP64 && (e = count_pattern_blocks(ctx, s, d_flags + 5)) != FE_OK)
         return fail(e);
-    cudaMemcpyAsync(h + 32, d_counts, 20 * sizeof(int), cudaMemcpyDeviceToHost, st);
-    cudaError_t ce = cudaStreamSynchronize(st);
+    cudaMemcpyAsync(h + 24, d_total, 28 * sizeof(int), cudaMemcpyDeviceToHost, st);  // totals, counts, flags
+    const cudaError_t ce = cudaStreamSynchronize(st);
     if (ce != cudaSuccess) {
-        set_error("row patterns: %s", cudaGetErrorString(ce));
+        set_error("row classes and patterns: %s", cudaGetErrorString(ce));
         return fail(FE_ERR_CUDA);
     }
     const unsigned long long* hc = (const unsigned long long*)(h + 32);
@@ -597,33 +618,6 @@ fe_status fe_assemble(fe_ctx* ctx, const fe_mesh* m, double freq_hz, int32_t pre
         s->n_dict = precision != FE_PREC_FP64 && !h[46] && h[45] <= kMaxDict ? h[45] : 0;
         *out = s;
         return FE_OK;
-    }
-    // Without patterns the products read the stored blocks, the class stencils
-    // and the block dictionary, and their rows are split by these costs, in
-    // units of one stored block of an explicit row: a general-stencil row
-    // costs 18 (complex64) or 27 (FP32 pairs, read through the block
-    // dictionary like an explicit row) such blocks, a diagonal-stencil row 10
-    // or 9 (per-CTA product times measured on GB300 and fitted to these three
-    // row kinds).  The third prefix counts the stored blocks of explicit rows
-    // only: a solve CTA packs its explicit rows' values at 9 times that prefix.
-    const int weights[3][3] = {{1, 18, 10}, {1, 27, 9}, {1, 0, 0}};
-    DevBuf* bufs[3] = {&s->cost_prefix, &s->cost_prefix_alu, &s->expl_prefix};
-    int* d_total = (int*)ctx->small.ptr + 24;
-    for (int k = 0; k < 3; ++k) {
-        if ((e = dev_alloc(st, *bufs[k], (size_t)(m->n_act + 1) * sizeof(int))) != FE_OK) return fail(e);
-        int* cp = (int*)bufs[k]->ptr;
-        k_row_cost<<<(unsigned)((m->n_act + 255) / 256), 256, 0, st>>>(
-            (const signed char*)s->row_class.ptr, (const StencilSet*)s->stencil.ptr, (const int*)m->row_ptr.ptr,
-            m->n_act, weights[k][0], weights[k][1], weights[k][2], cp);
-        count_launches(1);
-        if ((e = scan_exclusive(st, cp, cp, m->n_act, d_total + k, ctx->scan_tmp)) != FE_OK) return fail(e);
-        cudaMemcpyAsync(cp + m->n_act, d_total + k, sizeof(int), cudaMemcpyDeviceToDevice, st);
-    }
-    cudaMemcpyAsync(h + 24, d_total, 2 * sizeof(int), cudaMemcpyDeviceToHost, st);
-    ce = cudaStreamSynchronize(st);
-    if (ce != cudaSuccess) {
-        set_error("regular-row classes: %s", cudaGetErrorString(ce));
-        return fail(FE_ERR_CUDA);
     }
     s->cost_total = h[24];
     s->cost_total_alu = h[25];
