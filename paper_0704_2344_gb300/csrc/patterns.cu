@@ -230,6 +230,7 @@ __global__ void __launch_bounds__(96) k_pat_terms(const int* __restrict__ first_
         if (lane < 27) {
             const double w = al == 0 ? v[0].x : (al == 1 ? v[1].x : v[2].x);
             put(lane, w, pack_code(line, 3 * dx + al));
+            put(27 + (lane == 13 ? 26 : lane - (lane > 13)), w, pack_code(line, 3 * dx + al));  // own entry last
         }
     } else {
         if (lane < nb) {

@@ -20,7 +20,8 @@
 //
 // A pattern whose 27 blocks are real diagonal ones (the homogeneous interior)
 // is stored in full, 27 steps in the order of the grid, and read without the
-// term codes.
+// term codes; the same 27 follow once more with the row's own node last, for
+// kernels that read them by their codes.
 #pragma once
 
 #include "krylov.cuh"
