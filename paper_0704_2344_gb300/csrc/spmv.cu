@@ -356,8 +356,8 @@ static void launch_spmv_warp(int R, unsigned blocks, cudaStream_t st, const C* v
 // and tables instead of 1.1 GB of blocks.  Work items are (row, component,
 // column), consecutive lanes taking consecutive vector entries.  Four forms:
 //
-//   split   few items (below kSplitItems): 2 to 8 lanes share one, so that the
-//           chip's lanes are used and a lane's chain of dependent loads is short;
+//   split   few items: 2 to 8 lanes share one, so that the chip's lanes are used
+//           and a lane's chain of dependent loads is short;
 //   plain   one lane per item; the first blocks take the explicit rows
 //           (collected in a list, so that a warp holds rows of like length),
 //           the others sweep all rows for the real diagonal ones.  FP64 and
@@ -370,13 +370,14 @@ static void launch_spmv_warp(int R, unsigned blocks, cudaStream_t st, const C* v
 //           entries along a grid line.  Walking a range keeps a row's lines in
 //           L1 for the rows above and beside it.
 //
+// product_form says which sizes take which form, or the stored blocks.
 // Measured per product, from the stored blocks and here (in brackets: all by
-// the plain form): FP32 pairs, 9 261 rows 10.1 and 4.9 us (9.1); complex64,
+// the plain form): FP32 pairs, 9 261 rows 10.1 and 4.1 us (9.1); complex64,
 // 80^3 aircraft 196 and 28.9 us (32.4), 60^3 aircraft with 16 columns 306 and
 // 128 us (149); complex128, 48^3 nodes with 3 columns 840 and 106 us, 0.8 of
 // the FP64 pipe's rate on the non-zero terms.
 // ---------------------------------------------------------------------------
-template <typename C, int R_>
+template <typename C>
 __device__ __forceinline__ void pat_item(const PatView<C>& V, const C* __restrict__ x, C* __restrict__ y, int row,
                                          int al, int R, int c, bool want_diag) {
     const int4 t = __ldg(V.row + row);
@@ -400,8 +401,8 @@ __global__ void __launch_bounds__(256) k_spmv_pat(PatView<C> V, int n_rows, cons
     const int64_t d = e / R;
     const int c = (int)(e - d * R), i = (int)(d / 3), al = (int)(d - 3 * (int64_t)i);
     if (i >= (expl ? n_expl : n_rows)) return;
-    if (expl) pat_item<C, R_>(V, x, y, __ldg(list + i), al, R, c, false);
-    else pat_item<C, R_>(V, x, y, i, al, R, c, true);
+    if (expl) pat_item<C>(V, x, y, __ldg(list + i), al, R, c, false);
+    else pat_item<C>(V, x, y, i, al, R, c, true);
 }
 
 // split: K lanes per item, K R columns (a power of two up to 32) per warp part.
@@ -467,7 +468,7 @@ __global__ void __launch_bounds__(kKeepThreads, 1) k_spmv_pat_keep(PatView<float
     // explicit rows of this block, one walk beside the other
     const int e0 = (int)((int64_t)blockIdx.x * n_expl / gridDim.x), e1 = (int)((int64_t)(blockIdx.x + 1) * n_expl / gridDim.x);
     for (int i = e0 + (int)threadIdx.x / (3 * R); i < e1; i += step)
-        pat_item<float2, R>(V, x, y, __ldg(list + i), al, R, c, false);
+        pat_item<float2>(V, x, y, __ldg(list + i), al, R, c, false);
     const int r0 = (int)((int64_t)blockIdx.x * n_rows / gridDim.x), r1 = (int)((int64_t)(blockIdx.x + 1) * n_rows / gridDim.x);
     float w[27];
     int held = -1;
@@ -512,7 +513,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_spmv_pat_tile(PatView<float
     const int e0 = (int)((int64_t)blockIdx.x * n_expl / gridDim.x), e1 = (int)((int64_t)(blockIdx.x + 1) * n_expl / gridDim.x);
     for (int q = threadIdx.x; q < (e1 - e0) * 3 * R; q += kTileThreads) {
         const int c = q % R, d = q / R;
-        pat_item<float2, R>(V, x, y, __ldg(list + e0 + d / 3), d % 3, R, c, false);
+        pat_item<float2>(V, x, y, __ldg(list + e0 + d / 3), d % 3, R, c, false);
     }
     const int n4 = (n_rows + 3) / 4;
     const int q0 = (int)((int64_t)blockIdx.x * n4 / gridDim.x), q1 = (int)((int64_t)(blockIdx.x + 1) * n4 / gridDim.x);
@@ -524,7 +525,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_spmv_pat_tile(PatView<float
             tile = __ldg(V.id + r0 + 1) == id0 && __ldg(V.id + r0 + 2) == id0 && __ldg(V.id + r0 + 3) == id0 &&
                    __ldg(V.node_id + r0 + 3) - __ldg(V.node_id + r0) == 3;
         if (!tile) {
-            for (int row = r0; row < min(r0 + 4, n_rows); ++row) pat_item<float2, R>(V, x, y, row, al, R, c, true);
+            for (int row = r0; row < min(r0 + 4, n_rows); ++row) pat_item<float2>(V, x, y, row, al, R, c, true);
             continue;
         }
         const int4 t = __ldg(V.tab + id0);
@@ -560,10 +561,48 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_spmv_pat_tile(PatView<float
     }
 }
 
-// Items below which lanes share them: about half of the chip's resident
-// threads (152 SMs x 2048); items from which the walks, with one or a quarter
-// of an item per lane and step, have work for their 117 000 or 156 000 lanes.
-constexpr int64_t kSplitItems = 150000, kKeepItems = 300000, kTileItems = 600000;
+// Form of a product of `rows` rows and R columns on `lanes` resident lanes
+// (2 048 per SM, 311 296), by its items n = 3 rows R.  Lanes share an item while
+// that does not take more than the chip's: 8 up to n = lanes / 8, 4 up to
+// lanes / 4, 2 up to lanes / 2.  FP64 and FP32 pairs are plain above, and so is
+// complex64 of 8 columns and more until the tiles pay at n = 8 lanes; with up
+// to 4 columns complex64 keeps its weights.  Times in us per product in a
+// stream of them, on either side of a bound (cubes with a slab and a PEC body):
+//   keep    1 column 50 528 rows 12.4 shared and 14.4, 59 194 rows 14.5 and 14.4;
+//           2 columns 24 362 rows 12.3 and 14.4, 29 727 rows 14.4 and 14.4;
+//           4 columns 12 159 rows 12.3 and 14.4, 13 816 rows 14.4 and 14.4
+//   tile    8 columns 90 909 rows 50.3 plain and 49.3, 148 534 rows 75.9 and 67.8;
+//           16: 46 592 rows 53.2 and 55.1, 54 747 rows 59.5 and 55.8;
+//           32: 21 925 rows 52.1 and 50.1, 29 727 rows 65.7 and 63.5
+//           and 8 columns up to n = 2 lanes: 15 598 rows 20.5 and 18.5, 24 362 rows
+//           22.4 and 20.6, 26 973 rows 22.6 and 26.2
+// The stored blocks of a small system stay in L2, and a warp reads a row's
+// blocks at once, so that their chain of dependent loads is one shorter than a
+// pattern's (row, line, term, entry).  They round more (complex64 of 8 columns
+// and more 1.0e-7 against 4.6e-8), so they are taken only where the patterns
+// are clearly slower:
+//   complex64  1 column n <= lanes / 9: 10 640 rows 6.5 stored and 8.2, 12 159 8.2 and 8.2
+//              2 columns n <= lanes / 5: 9 253 rows 8.2 and 8.3, 10 640 8.3 and 8.3
+//              8 and 16 columns from lanes / 2 to 4/5 lanes, between the shared
+//              items and the others: 8 columns 9 253 rows 12.4 and 16.4; 16 columns
+//              4 912 rows 14.4 and 18.5
+//   FP32 pairs 1 and 4 columns n <= lanes / 32: 2 196 rows 6.2 and 8.0, 3 374 8.2 and
+//              7.3; 4 columns 512 rows 6.3 and 6.7, 1 331 8.2 and 8.2
+enum class Form { kStored, kSplit8, kSplit4, kSplit2, kPlain, kWalk };
+
+static Form product_form(int precision, int64_t rows, int R, int sms) {
+    const double n = 3.0 * (double)rows * R, lanes = 2048.0 * sms;
+    if (R > 32 || (R & (R - 1))) return Form::kPlain;
+    const bool c64 = precision == FE_PREC_MIXED;
+    if (c64 && ((R == 1 && 9 * n <= lanes) || (R == 2 && 5 * n <= lanes) ||
+                ((R == 8 || R == 16) && 2 * n > lanes && 5 * n <= 4 * lanes)))
+        return Form::kStored;
+    if (precision == FE_PREC_DF && (R == 1 || R == 4) && 32 * n <= lanes) return Form::kStored;
+    if (8 * R <= 32 && 8 * n <= lanes) return Form::kSplit8;
+    if (4 * R <= 32 && 4 * n <= lanes) return Form::kSplit4;
+    if (2 * R <= 32 && 2 * n <= lanes) return Form::kSplit2;
+    return c64 && (R <= 4 || (R == 8 && n <= 2 * lanes) || n > 8 * lanes) ? Form::kWalk : Form::kPlain;
+}
 
 template <typename C, int R>
 static void launch_pat_plain(cudaStream_t st, const PatView<C>& V, const fe_system* s, int nrhs, const C* x, C* y) {
@@ -573,71 +612,53 @@ static void launch_pat_plain(cudaStream_t st, const PatView<C>& V, const fe_syst
 }
 
 template <typename C, int R>
-static void launch_pat_r(cudaStream_t st, const PatView<C>& V, const fe_system* s, int sms, const C* x, C* y) {
+static void launch_pat_r(cudaStream_t st, const PatView<C>& V, const fe_system* s, int sms, Form form, const C* x,
+                         C* y) {
     const int n = s->mesh->n_act;
     const int64_t items = (int64_t)n * 3 * R;
     auto blocks = [&](int k) { return (unsigned)((items * k + 255) / 256); };
     if constexpr (8 * R <= 32)
-        if (8 * items <= 2 * kSplitItems) {
+        if (form == Form::kSplit8) {
             k_spmv_pat_split<C, R, 8><<<blocks(8), 256, 0, st>>>(V, n, x, y);
             return;
         }
     if constexpr (4 * R <= 32)
-        if (4 * items <= 2 * kSplitItems) {
+        if (form == Form::kSplit4) {
             k_spmv_pat_split<C, R, 4><<<blocks(4), 256, 0, st>>>(V, n, x, y);
             return;
         }
     if constexpr (2 * R <= 32)
-        if (items <= kSplitItems) {
+        if (form == Form::kSplit2) {
             k_spmv_pat_split<C, R, 2><<<blocks(2), 256, 0, st>>>(V, n, x, y);
             return;
         }
-    if constexpr (std::is_same<C, float2>::value && R <= 4)
-        if (items >= kKeepItems) {
-            k_spmv_pat_keep<R><<<sms, kKeepThreads, 0, st>>>(V, n, (const int*)s->pat_list.ptr, s->n_expl, x, y);
-            return;
-        }
-    if constexpr (std::is_same<C, float2>::value && R >= 8)
-        if (items >= kTileItems) {
-            k_spmv_pat_tile<R><<<sms, kTileThreads, 0, st>>>(V, n, (const int*)s->pat_list.ptr, s->n_expl, x, y);
+    if constexpr (std::is_same<C, float2>::value)
+        if (form == Form::kWalk) {
+            if constexpr (R <= 4)
+                k_spmv_pat_keep<R><<<sms, kKeepThreads, 0, st>>>(V, n, (const int*)s->pat_list.ptr, s->n_expl, x, y);
+            else
+                k_spmv_pat_tile<R><<<sms, kTileThreads, 0, st>>>(V, n, (const int*)s->pat_list.ptr, s->n_expl, x, y);
             return;
         }
     launch_pat_plain<C, R>(st, V, s, R, x, y);
 }
 
 template <typename C>
-static void launch_spmv_pat(cudaStream_t st, const fe_system* s, int sms, const void* terms, int nrhs, const C* x,
-                            C* y) {
+static void launch_spmv_pat(cudaStream_t st, const fe_system* s, int sms, const void* terms, int nrhs, Form form,
+                            const C* x, C* y) {
     const fe_mesh* m = s->mesh;
     const PatView<C> V{(const uint16_t*)s->pat_id.ptr, (const int4*)s->pat_row.ptr, (const int4*)s->pat_tab.ptr, (const C*)terms,
                        (const int*)m->node_id.ptr,     (const int*)m->node_rank.ptr, m->nx + 1,
                        (m->nx + 1) * (m->ny + 1)};
     switch (nrhs) {
-        case 1: launch_pat_r<C, 1>(st, V, s, sms, x, y); break;
-        case 2: launch_pat_r<C, 2>(st, V, s, sms, x, y); break;
-        case 4: launch_pat_r<C, 4>(st, V, s, sms, x, y); break;
-        case 8: launch_pat_r<C, 8>(st, V, s, sms, x, y); break;
-        case 16: launch_pat_r<C, 16>(st, V, s, sms, x, y); break;
-        case 32: launch_pat_r<C, 32>(st, V, s, sms, x, y); break;
+        case 1: launch_pat_r<C, 1>(st, V, s, sms, form, x, y); break;
+        case 2: launch_pat_r<C, 2>(st, V, s, sms, form, x, y); break;
+        case 4: launch_pat_r<C, 4>(st, V, s, sms, form, x, y); break;
+        case 8: launch_pat_r<C, 8>(st, V, s, sms, form, x, y); break;
+        case 16: launch_pat_r<C, 16>(st, V, s, sms, form, x, y); break;
+        case 32: launch_pat_r<C, 32>(st, V, s, sms, form, x, y); break;
         default: launch_pat_plain<C, 0>(st, V, s, nrhs, x, y); break;
     }
-}
-
-// Products so small that neither the lanes nor the bandwidth bound them: the
-// patterns' chain of dependent loads (row, table, line, term, entry) is one
-// longer than the stored blocks', which stay in L2.  Measured per call:
-// complex64, 1 column, 9 261 rows 8.2 us by patterns and 6.2 stored, equal at
-// 15 625 rows; 2 columns, 5 832 rows 8.2 and 6.2; 4 columns and more, patterns
-// are ahead from the start, but for 8 and 16 between the range where two lanes
-// share an item and the one that fills the lanes (8 columns, 9 261 rows 14.4 and
-// 12.3; 5 832 rows 10.4 and 12.3, 15 625 rows 14.4 and 18.5).  FP32 pairs,
-// 2 197 rows: 1 column 8.2 and 6.2, 4 columns 10.3 and 9.2; equal at 4 096 rows.
-// FP64 is ahead at every size.
-static bool small_stored(int precision, int n_rows, int nrhs) {
-    const int64_t items = (int64_t)n_rows * 3 * nrhs;
-    if (precision == FE_PREC_MIXED)
-        return nrhs <= 2 ? n_rows <= 9300 : (nrhs == 8 || nrhs == 16) && items > kSplitItems && items <= 240000;
-    return precision == FE_PREC_DF && (nrhs <= 2 || nrhs == 4) && n_rows <= 2200;
 }
 
 }  // namespace fe
@@ -664,13 +685,14 @@ fe_status fe_spmv(fe_ctx* ctx, const fe_system* s, int32_t precision, int32_t nr
                         : precision == FE_PREC_MIXED ? s->pat_t32.ptr
                         : precision == FE_PREC_DF ? s->pat_tdf.ptr : nullptr;
     const int64_t pat_blocks = ((int64_t)m->n_act + s->n_expl) * 3 * nrhs / 256 + 2;
-    if (s->n_pat && terms && pat_blocks < (1ll << 31) && !small_stored(precision, m->n_act, nrhs)) {
+    const Form form = product_form(precision, m->n_act, nrhs, ctx->num_sms);
+    if (s->n_pat && terms && pat_blocks < (1ll << 31) && form != Form::kStored) {
         if (precision == FE_PREC_FP64)
-            launch_spmv_pat<double2>(st, s, ctx->num_sms, terms, nrhs, (const double2*)x, (double2*)y);
+            launch_spmv_pat<double2>(st, s, ctx->num_sms, terms, nrhs, form, (const double2*)x, (double2*)y);
         else if (precision == FE_PREC_MIXED)
-            launch_spmv_pat<float2>(st, s, ctx->num_sms, terms, nrhs, (const float2*)x, (float2*)y);
+            launch_spmv_pat<float2>(st, s, ctx->num_sms, terms, nrhs, form, (const float2*)x, (float2*)y);
         else
-            launch_spmv_pat<float4>(st, s, ctx->num_sms, terms, nrhs, (const float4*)x, (float4*)y);
+            launch_spmv_pat<float4>(st, s, ctx->num_sms, terms, nrhs, form, (const float4*)x, (float4*)y);
     } else if (precision == FE_PREC_FP64) {
         if (pow2 && nrhs >= 8)
             launch_spmm_rows<double2>(nrhs, st, ctx->num_sms, (const double2*)s->val64.ptr, s->stride, col, rp,
