@@ -218,6 +218,12 @@ typedef struct fe_system_stats {
     int64_t device_bytes;      /* device memory held by the system */
 } fe_system_stats;
 fe_status fe_system_info(const fe_system* s, fe_system_stats* out);
+/* Row patterns of a system: how many it has (0: none, its products and solves
+ * read the stored blocks) and, optionally, the terms of one product over all
+ * rows and components, padding included (a term is one real weight times a
+ * complex vector entry; 0 without patterns).  Waits for the context's stream
+ * when terms is asked for.  Errors: FE_ERR_INVALID_ARG (NULL), FE_ERR_CUDA. */
+fe_status fe_system_patterns(fe_ctx* ctx, const fe_system* s, int32_t* n_patterns, int64_t* terms);
 /* Copies the FP32-pair values of a system assembled with FE_PREC_DF to a
  * caller-allocated HOST buffer vals_df[nnzb*9*4 floats]: per entry
  * (re_hi, im_hi, re_lo, im_lo), block-major as vals_c128.  Errors:

@@ -631,6 +631,24 @@ fe_status fe_assemble(fe_ctx* ctx, const fe_mesh* m, double freq_hz, int32_t pre
     return FE_OK;
 }
 
+fe_status fe_system_patterns(fe_ctx* ctx, const fe_system* s, int32_t* n_patterns, int64_t* terms) {
+    if (!ctx || !s || !n_patterns) {
+        set_error("fe_system_patterns: NULL argument");
+        return FE_ERR_INVALID_ARG;
+    }
+    *n_patterns = s->n_pat;
+    if (!terms) return FE_OK;
+    *terms = 0;
+    if (!s->n_pat) return FE_OK;
+    std::vector<int4> tab(s->n_pat);
+    std::vector<uint16_t> id(s->mesh->n_act);
+    FE_CUDA(cudaMemcpyAsync(tab.data(), s->pat_tab.ptr, tab.size() * sizeof(int4), cudaMemcpyDeviceToHost, ctx->stream));
+    FE_CUDA(cudaMemcpyAsync(id.data(), s->pat_id.ptr, id.size() * sizeof(uint16_t), cudaMemcpyDeviceToHost, ctx->stream));
+    FE_CUDA(cudaStreamSynchronize(ctx->stream));
+    for (uint16_t p : id) *terms += 3 * (int64_t)(tab[p].y + tab[p].z);
+    return FE_OK;
+}
+
 fe_status fe_system_info(const fe_system* s, fe_system_stats* out) {
     if (!s || !out) {
         set_error("fe_system_info: NULL argument");

@@ -140,6 +140,7 @@ def load() -> C.CDLL:
         "fe_system_factor_bicp": (C.c_int, [P, P, C.c_int32]),
         "fe_system_export_bicp": (C.c_int, [P, P, P, P]),
         "fe_system_info": (C.c_int, [P, C.POINTER(fe_system_stats)]),
+        "fe_system_patterns": (C.c_int, [P, P, C.POINTER(C.c_int32), C.POINTER(C.c_int64)]),
         "fe_system_destroy": (None, [P]),
         "fe_rhs": (C.c_int, [P, P, C.c_int32, C.POINTER(fe_planewave), P, C.c_int32]),
         "fe_spmv": (C.c_int, [P, P, C.c_int32, C.c_int32, P, P]),
@@ -327,6 +328,13 @@ def fe_system_info(system) -> dict:
     st = fe_system_stats()
     _check(load().fe_system_info(system, C.byref(st)), "fe_system_info")
     return {n: int(getattr(st, n)) for n, _ in fe_system_stats._fields_}
+
+
+def fe_system_patterns(ctx, system) -> tuple[int, int]:
+    """(row patterns of the system, 0 without; terms of one product)."""
+    n, terms = C.c_int32(0), C.c_int64(0)
+    _check(load().fe_system_patterns(ctx, system, C.byref(n), C.byref(terms)), "fe_system_patterns")
+    return int(n.value), int(terms.value)
 
 
 def fe_system_export_df(ctx, system, mesh) -> np.ndarray:
