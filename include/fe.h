@@ -441,8 +441,8 @@ fe_status fe_solve_rhs_noalloc(fe_ctx* ctx, const fe_system* s, int32_t nrhs, co
  * each admitted request's mesh, system (Eqs. 1-4) and right-hand sides.
  * Solves then run in segments of about 25 ms: each segment is one
  * persistent cooperative launch per right-hand-side tile width (1, 2, 4, 8,
- * 16 or 32 after padding with zero columns), the widths side by side on
- * their own streams; every request has its own range of CTAs, synchronises
+ * 16 or 32 after padding with zero columns) and kind of system (with or
+ * without row patterns), side by side on their own streams; every request has its own range of CTAs, synchronises
  * only among them, and keeps its Krylov state on the device from segment to
  * segment.  Between segments finished requests are handed out and their
  * memory freed, and requests that arrived meanwhile are admitted and start
@@ -493,7 +493,7 @@ typedef struct fe_result {
 
 typedef struct fe_serve_stats {
     int64_t submitted, completed, failed;
-    int64_t launches;           /* persistent solve launches (one per tile width per segment) */
+    int64_t launches;           /* persistent solve launches (one per tile width and kind of system per segment) */
     int64_t jobs_launched;      /* requests summed over segments */
     int64_t budget_bytes;       /* admission budget */
     int64_t peak_admitted_bytes;/* largest sum of admitted estimates */

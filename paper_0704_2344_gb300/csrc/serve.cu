@@ -1,7 +1,7 @@
 // Serving: a request queue solved with continuous batching.
 //
 // A worker thread owns an internal context (its own stream on the caller's
-// device) and one more stream per right-hand-side tile width.  Solves run in
+// device) and two more streams per right-hand-side tile width.  Solves run in
 // segments: a persistent multi-system launch advances each of its requests
 // by at most seg_iters iterations and saves their Krylov state on the device
 // (solve_kernels.cuh, JobState).  Each loop turn the worker
@@ -12,8 +12,9 @@
 //   2. plans the segment with fe_serve_plan over all active requests: every
 //      request has a CTA count fixed by its own size, and requests run in
 //      arrival order while their counts fit the device;
-//   3. starts one cooperative launch per tile width, each on its own stream,
-//      so that widths run side by side on disjoint SMs, and waits for them;
+//   3. starts one cooperative launch per tile width and kind of system (with or
+//      without row patterns, which run different kernels), each on its own
+//      stream, so that they run side by side on disjoint SMs, and waits for them;
 //   4. hands out the requests that finished and frees their memory.
 // A request submitted meanwhile is admitted at the next turn, a few
 // milliseconds later, and runs beside the requests already in flight.
@@ -36,6 +37,7 @@ fe_status job_create(fe_ctx* ctx, const fe_system* s, int nrhs, const double2* d
                      SolveJob** out);
 int job_width(const SolveJob* j);
 int64_t job_rows(const SolveJob* j);
+bool job_has_patterns(const SolveJob* j);
 void job_destroy(fe_ctx* ctx, SolveJob* j);
 fe_status jobs_launch(fe_ctx* ctx, SolveJob* const* jobs, const int* n_cta, int n, cudaStream_t stream,
                       const int* seg_iters);
@@ -104,10 +106,13 @@ int segment_iters(const fe_serve_opts& o, const ServeReq* q, bool alone, int wid
     return (int)std::max(16.0, std::min(1e6, kSegTargetMs / ms));
 }
 
-int width_slot(int width) {
+// One launch each: the requests of one tile width (1 to 32), with or without
+// row patterns.
+constexpr int kSlots = 12;
+int launch_slot(const SolveJob* j) {
     int k = 0;
-    while ((1 << k) < width && k < 5) ++k;
-    return k;
+    while ((1 << k) < job_width(j) && k < 5) ++k;
+    return job_has_patterns(j) ? k : 6 + k;
 }
 
 int tile_width(int nrhs) {
@@ -153,7 +158,7 @@ struct fe_server {
     std::condition_variable cv_work, cv_done;
     std::deque<ServeReq*> queue;                  // submitted, not admitted
     std::vector<ServeReq*> ready;                 // admitted and built, in arrival order (worker only)
-    cudaStream_t wstream[6] = {};                 // one launch stream per tile width 1..32
+    cudaStream_t wstream[kSlots] = {};            // one launch stream per slot
     std::unordered_map<uint64_t, ServeReq*> all;  // every unreleased ticket
     uint64_t next_ticket = 1;
     bool stop = false;
@@ -269,14 +274,14 @@ bool worker_turn(fe_server* S) {
     // while a large one runs find CTAs beside it
     const int max_job = S->o.max_job_ctas > 0 ? std::min(S->o.max_job_ctas, max_ctas) : std::max(1, max_ctas * 3 / 4);
     fe_serve_plan(n, rows.data(), width.data(), max_ctas, max_job, S->o.work_per_cta, n_cta.data());
-    std::vector<SolveJob*> jobs[6];
-    std::vector<int> ctas[6], iters[6];
-    std::vector<ServeReq*> in_seg[6];
+    std::vector<SolveJob*> jobs[kSlots];
+    std::vector<int> ctas[kSlots], iters[kSlots];
+    std::vector<ServeReq*> in_seg[kSlots];
     int n_seg = 0;
     const bool alone = n == 1;
     for (int i = 0; i < n; ++i) {
         if (n_cta[i] <= 0) continue;
-        const int k = width_slot(width[i]);
+        const int k = launch_slot(S->ready[i]->job);
         jobs[k].push_back(S->ready[i]->job);
         ctas[k].push_back(n_cta[i]);
         iters[k].push_back(segment_iters(S->o, S->ready[i], alone, width[i], n_cta[i]));
@@ -286,15 +291,21 @@ bool worker_turn(fe_server* S) {
     const auto t_seg0 = Clock::now();
     fe_status e = FE_OK;
     int launched = 0;
-    for (int k = 0; k < 6 && e == FE_OK; ++k) {
+    for (int k = 0; k < kSlots && e == FE_OK; ++k) {
         if (jobs[k].empty()) continue;
+        if (!S->wstream[k] && cudaStreamCreateWithFlags(&S->wstream[k], cudaStreamNonBlocking) != cudaSuccess) {
+            S->wstream[k] = nullptr;
+            set_error("serve: stream creation failed");
+            e = FE_ERR_CUDA;
+            break;
+        }
         e = jobs_launch(S->ictx, jobs[k].data(), ctas[k].data(), (int)jobs[k].size(), S->wstream[k],
                         iters[k].data());
         if (e == FE_OK) ++launched;
     }
     std::string launch_msg = e == FE_OK ? std::string() : std::string(fe_last_error());
-    for (int k = 0; k < 6; ++k) {
-        if (jobs[k].empty()) continue;
+    for (int k = 0; k < kSlots; ++k) {
+        if (jobs[k].empty() || !S->wstream[k]) continue;
         const cudaError_t ce = cudaStreamSynchronize(S->wstream[k]);
         if (ce != cudaSuccess && e == FE_OK) {
             e = FE_ERR_CUDA;
@@ -310,7 +321,7 @@ bool worker_turn(fe_server* S) {
     // hand out what finished; the rest stays for the next segment
     std::vector<ServeReq*> keep;
     for (ServeReq* q : S->ready) {
-        const int k = width_slot(job_width(q->job));
+        const int k = launch_slot(q->job);
         bool ran = false;
         for (size_t i = 0; i < in_seg[k].size(); ++i)
             if (in_seg[k][i] == q) {
@@ -475,7 +486,7 @@ fe_status fe_serve_create(fe_ctx* ctx, const fe_serve_opts* opt, fe_server** out
         return FE_ERR_CUDA;
     }
     S->stats.budget_bytes = o.hbm_budget > 0 ? o.hbm_budget : (int64_t)(free_b / 10 * 8);
-    for (int k = 0; k < 6; ++k)
+    for (int k = 0; k < 6; ++k)  // the others when first used: few streams have such requests
         if (cudaStreamCreateWithFlags(&S->wstream[k], cudaStreamNonBlocking) != cudaSuccess) {
             set_error("fe_serve_create: stream creation failed");
             for (int q = 0; q < k; ++q) cudaStreamDestroy(S->wstream[q]);
@@ -621,7 +632,7 @@ void fe_serve_destroy(fe_server* S) {
     }
     for (auto& kv : S->all) delete kv.second;
     cudaStreamSynchronize(S->ictx->stream);
-    for (int k = 0; k < 6; ++k)
+    for (int k = 0; k < kSlots; ++k)
         if (S->wstream[k]) cudaStreamDestroy(S->wstream[k]);
     fe_ctx_destroy(S->ictx);
     delete S;

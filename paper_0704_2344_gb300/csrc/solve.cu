@@ -554,6 +554,7 @@ fe_status job_create(fe_ctx* ctx, const fe_system* s, int nrhs, const double2* d
 
 int job_width(const SolveJob* j) { return j->R; }
 int64_t job_rows(const SolveJob* j) { return j->P.n_rows; }
+bool job_has_patterns(const SolveJob* j) { return j->P.pat_id != nullptr; }  // which kernels run it
 
 void job_destroy(fe_ctx* ctx, SolveJob* j) {
     if (!j) return;
@@ -561,8 +562,8 @@ void job_destroy(fe_ctx* ctx, SolveJob* j) {
     delete j;
 }
 
-// Enqueues one cooperative launch of n jobs of one width and precision on
-// `stream`; job i gets n_cta[i] CTAs (1..its row count) and runs at most
+// Enqueues one cooperative launch of n jobs of one width and precision, all
+// with or all without row patterns, on `stream`; job i gets n_cta[i] CTAs (1..its row count) and runs at most
 // seg_iters[i] iterations (seg_iters NULL or 0: to the end), resuming where
 // its last launch stopped.  A job must keep its CTA count from launch to launch: the CTAs
 // own its vector rows.
@@ -571,10 +572,11 @@ fe_status jobs_launch(fe_ctx* ctx, SolveJob* const* jobs, const int* n_cta, int 
     if (n < 1) return FE_OK;
     const int R = jobs[0]->R;
     const int prec = jobs[0]->prec;
+    const bool pat = job_has_patterns(jobs[0]);
     int64_t total = 0;
     for (int i = 0; i < n; ++i) {
-        if (jobs[i]->R != R || jobs[i]->prec != prec) {
-            set_error("jobs: one launch takes one tile width and one precision");
+        if (jobs[i]->R != R || jobs[i]->prec != prec || job_has_patterns(jobs[i]) != pat) {
+            set_error("jobs: one launch takes one tile width, one precision and one kind of system");
             return FE_ERR_INVALID_ARG;
         }
         if (n_cta[i] < 1 || n_cta[i] > std::max(1, jobs[i]->P.n_rows)) {
@@ -587,25 +589,11 @@ fe_status jobs_launch(fe_ctx* ctx, SolveJob* const* jobs, const int* n_cta, int 
         set_error("jobs: %lld CTAs exceed one per SM", (long long)total);
         return FE_ERR_INVALID_ARG;
     }
-    // systems with and without row patterns run different kernels, one after
-    // the other on the stream
-    for (int pat = 1; pat >= 0; --pat) {
-        std::vector<SolveJob*> js;
-        std::vector<int> ctas, segs;
-        for (int i = 0; i < n; ++i)
-            if ((jobs[i]->P.pat_id != nullptr) == (pat == 1)) {
-                js.push_back(jobs[i]);
-                ctas.push_back(n_cta[i]);
-                segs.push_back(seg_iters ? seg_iters[i] : 0);
-            }
-        if (js.empty()) continue;
-        FE_TRY(with_inner_type(prec, [&](auto* tag) {
-            using T = std::remove_pointer_t<decltype(tag)>;
-            return pat ? launch_pat_jobs<T>(ctx, R, js.data(), ctas.data(), (int)js.size(), stream, segs.data())
-                       : launch_jobs_w<T>(ctx, R, js.data(), ctas.data(), (int)js.size(), stream, segs.data());
-        }));
-    }
-    return FE_OK;
+    return with_inner_type(prec, [&](auto* tag) {
+        using T = std::remove_pointer_t<decltype(tag)>;
+        return pat ? launch_pat_jobs<T>(ctx, R, jobs, n_cta, n, stream, seg_iters)
+                   : launch_jobs_w<T>(ctx, R, jobs, n_cta, n, stream, seg_iters);
+    });
 }
 
 // A job's progress after a launch, from its state block: whether the solve

@@ -115,3 +115,19 @@ def test_served_batch_of_both_kinds(fe, ctx, precision):
         maps = fem.mesh_maps(prob)
         A, B = fem.assemble(prob, maps=maps), fem.rhs(prob, waves, maps=maps)
         assert fem.true_relative_residual(A, r["x"], B).max() <= 1e-8
+
+
+def test_both_kinds_run_side_by_side(fe, ctx):
+    """Requests of one tile width with and without patterns are launched separately in a segment, not one after the
+    other in one launch's turn: two requests that share every segment make two launches of it."""
+    srv = fe.fe_serve_create(ctx, fe.serve_opts(seg_iters=16))
+    try:
+        probs = [_speckle(), W.pec_box_problem(9, 2.5e9, np.random.default_rng(0))]
+        waves = [W.random_waves(1, np.random.default_rng(q)) for q in range(2)]
+        tickets = [fe.fe_serve_submit(srv, p, w) for p, w in zip(probs, waves)]
+        results = [fe.fe_serve_wait(srv, t, timeout_s=60.0) for t in tickets]
+        info = fe.fe_serve_info(srv)
+    finally:
+        fe.fe_serve_destroy(srv)
+    assert all(r["status"] == 0 for r in results) and max(r["batch_jobs"] for r in results) == 2
+    assert info["launches"] == info["jobs_launched"]
