@@ -316,7 +316,8 @@ fe_status fe_spmv_half(fe_ctx* ctx, const fe_system* s, int32_t precision, int32
  * for every right-hand side.  Up to
  * rhs_tile right-hand sides are solved together in one persistent device
  * launch.  With rhs_tile = 0 and at least 8 right-hand sides, the first solve
- * of a system shape (unknowns, right-hand sides, precision, variant, device)
+ * of a system shape (unknowns, right-hand sides, precision, variant, device,
+ * with or without row patterns)
  * runs the autotuner: short trial launches (32 iterations of the first
  * columns) for every tile width in {8, 16, 32} up to the column count and
  * grids of all or three quarters of the SMs, timed with CUDA events; the

@@ -302,9 +302,10 @@ constexpr double kTuneTie = 0.05;
 struct TuneKey {
     int64_t n_dof, nnzb;
     int nrhs, prec, variant, device;
+    bool pat;  // which kernels the trials timed (row patterns or not)
     bool operator<(const TuneKey& o) const {
-        return std::tie(n_dof, nnzb, nrhs, prec, variant, device) <
-               std::tie(o.n_dof, o.nnzb, o.nrhs, o.prec, o.variant, o.device);
+        return std::tie(n_dof, nnzb, nrhs, prec, variant, device, pat) <
+               std::tie(o.n_dof, o.nnzb, o.nrhs, o.prec, o.variant, o.device, o.pat);
     }
 };
 static std::mutex g_tune_mu;
@@ -313,7 +314,7 @@ static std::map<TuneKey, std::pair<int, int>> g_tune;  // (tile width, CTAs)
 static fe_status autotune(fe_ctx* ctx, const fe_system* s, int nrhs, const double2* d_b, const fe_solve_opts& o,
                           int* R_out, int* cta_out, int* how, double* tune_ms) {
     const TuneKey key{3 * (int64_t)s->mesh->n_act, s->mesh->nnzb, std::min(nrhs, 32), o.precision, s->variant,
-                      ctx->device};
+                      ctx->device, s->n_pat > 0};
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         auto it = g_tune.find(key);

@@ -131,3 +131,23 @@ def test_both_kinds_run_side_by_side(fe, ctx):
         fe.fe_serve_destroy(srv)
     assert all(r["status"] == 0 for r in results) and max(r["batch_jobs"] for r in results) == 2
     assert info["launches"] == info["jobs_launched"]
+
+
+def test_tuned_choice_is_kept_per_kind_of_kernel(fe, ctx):
+    """Two systems of one shape, one with patterns and one without, run different kernels: each is tuned itself."""
+    rng = np.random.default_rng(8)
+    prob = _core(9, 7, seed=8)
+    flat = W.empty_box(9)
+    waves = W.random_waves(13, rng)
+    how = []
+    for p, has in ((flat, True), (prob, False), (flat, True), (prob, False)):
+        m, s = _system(fe, ctx, p, fe.FE_PREC_DF)
+        try:
+            assert (fe.fe_system_patterns(ctx, s)[0] > 0) == has
+            fe.fe_solve_batch(ctx, s, waves, fe.fe_mesh_info(m)["n_dof"], fe.solve_opts(max_iter=40),
+                              raise_on_fail=False)
+            how.append(fe.fe_last_solve_stats(ctx)["tuned"])
+        finally:
+            fe.fe_system_destroy(s)
+            fe.fe_mesh_destroy(m)
+    assert how == [1, 1, 2, 2]
