@@ -438,7 +438,8 @@ fe_status fe_solve_rhs_noalloc(fe_ctx* ctx, const fe_system* s, int32_t nrhs, co
  * the context passed to fe_serve_create (whose options, variant, abc_sigma
  * and penalty_s, apply to every request; that context stays free for the
  * caller).  The worker admits queued requests in arrival order while the
- * sum of their estimated device memory stays within the budget, and builds
+ * sum of their estimated device memory stays within the budget (a request that
+ * fits it only without row patterns is served without), and builds
  * each admitted request's mesh, system (Eqs. 1-4) and right-hand sides.
  * Solves then run in segments of about 25 ms: each segment is one
  * persistent cooperative launch per right-hand-side tile width (1, 2, 4, 8,

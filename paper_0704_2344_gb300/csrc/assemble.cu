@@ -445,13 +445,9 @@ static void system_free(fe_system* s) {
     s->n_dict = 0;
 }
 
-}  // namespace fe
-
-using namespace fe;
-
-extern "C" {
-
-fe_status fe_assemble(fe_ctx* ctx, const fe_mesh* m, double freq_hz, int32_t precision, fe_system** out) {
+// patterns false: none are built (a server whose budget they would not fit).
+fe_status assemble_system(fe_ctx* ctx, const fe_mesh* m, double freq_hz, int32_t precision, bool patterns,
+                          fe_system** out) {
     if (!ctx || !m || !out) {
         set_error("fe_assemble: NULL argument");
         return FE_ERR_INVALID_ARG;
@@ -536,7 +532,7 @@ fe_status fe_assemble(fe_ctx* ctx, const fe_mesh* m, double freq_hz, int32_t pre
         dev_free(st, row_group);
         return fail(e);
     };
-    if ((e = group_rows(ctx, s, row_group, d_flags)) != FE_OK) return fail_group(e);
+    if (patterns && (e = group_rows(ctx, s, row_group, d_flags)) != FE_OK) return fail_group(e);
     // one warp per block for the few first rows, so that each has an SM's FP64
     // pipe to itself (80 rows: 48 us in blocks of eight warps)
     const int threads = s->n_pat ? 32 : 256;
@@ -629,6 +625,16 @@ fe_status fe_assemble(fe_ctx* ctx, const fe_mesh* m, double freq_hz, int32_t pre
     if ((e = build_block_dict(ctx, s)) != FE_OK) return fail(e);
     *out = s;
     return FE_OK;
+}
+
+}  // namespace fe
+
+using namespace fe;
+
+extern "C" {
+
+fe_status fe_assemble(fe_ctx* ctx, const fe_mesh* m, double freq_hz, int32_t precision, fe_system** out) {
+    return assemble_system(ctx, m, freq_hz, precision, true, out);
 }
 
 fe_status fe_system_patterns(fe_ctx* ctx, const fe_system* s, int32_t* n_patterns, int64_t* terms) {

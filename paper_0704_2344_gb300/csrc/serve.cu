@@ -43,7 +43,9 @@ fe_status jobs_launch(fe_ctx* ctx, SolveJob* const* jobs, const int* n_cta, int 
                       const int* seg_iters);
 fe_status job_progress(SolveJob* j, cudaStream_t stream, bool* finished, int* seg_done, double* seg_ms);
 fe_status job_collect(fe_ctx* ctx, SolveJob* j, fe_complex* x_host, fe_solve_report* rep);
-size_t workspace_bytes(int64_t n_dof, int R, int prec, int max_cta, int64_t pk_entries);
+size_t workspace_bytes(int64_t n_dof, int R, int prec, int max_cta, int64_t pk_entries, bool pat);
+fe_status assemble_system(fe_ctx* ctx, const fe_mesh* m, double freq_hz, int32_t precision, bool patterns,
+                          fe_system** out);
 fe_status build_rhs(fe_ctx* ctx, const fe_system* s, int nrhs, const fe_planewave* waves, double2* d_B,
                     DevBuf& wave_buf);
 
@@ -60,6 +62,7 @@ struct ServeReq {
     std::vector<fe_planewave> waves;
     int width = 1;  // power-of-two tile width >= nrhs
     int64_t est_bytes = 0;
+    bool patterns = true;  // false: only its stored blocks fit the server's budget
     double t_submit = 0.0, t_admit = 0.0, t_done = 0.0;
     fe_mesh* mesh = nullptr;
     fe_system* sys = nullptr;
@@ -124,8 +127,10 @@ int tile_width(int nrhs) {
 // Upper bound of the device bytes a request holds while admitted: the mesh
 // maps, the block values (complex128, plus complex64 in the mixed mode), the
 // block-Jacobi inverses, the right-hand sides and the Krylov workspace, for
-// the worst case of every grid node active with 27 neighbours.
-int64_t estimate_bytes(const fe_mesh_desc& d, int nrhs, int width, int prec, int num_sms) {
+// the worst case of every grid node active with 27 neighbours.  The row
+// patterns add up to a quarter (as many as the mesh may have); a request that
+// fits the budget only without them is served from the stored blocks.
+int64_t estimate_bytes(const fe_mesh_desc& d, int nrhs, int width, int prec, int num_sms, bool patterns) {
     const int64_t n_el = (int64_t)d.nx * d.ny * d.nz;
     const int64_t nodes = (int64_t)(d.nx + 1) * (d.ny + 1) * (d.nz + 1);
     const int64_t nnzb = 27 * nodes;
@@ -135,11 +140,12 @@ int64_t estimate_bytes(const fe_mesh_desc& d, int nrhs, int width, int prec, int
     const int64_t per_entry = prec == FE_PREC_FP64 ? 16 : (prec == FE_PREC_MIXED ? 24 : 32);
     const int64_t sys = 9 * stride * per_entry + 9 * nodes * 24 + nodes * 13 + 65536;
     // row patterns: term lists, the row tables and what their construction holds
-    const int64_t pat = (int64_t)pat_limit(nodes) * kPatStride * 3 * per_entry + 80 * nodes + (1 << 18);
+    const int64_t pat =
+        patterns ? (int64_t)pat_limit(nodes) * kPatStride * 3 * per_entry + 80 * nodes + (1 << 18) : 0;
     const int64_t rhs = 3 * nodes * (int64_t)nrhs * 16;
     // the packed explicit rows of a single-column launch: at most every block
     const int64_t pk = (width == 1 && prec != FE_PREC_FP64) ? 9 * nnzb : 0;
-    const int64_t ws = (int64_t)workspace_bytes(3 * nodes, width, prec, 2 * num_sms, pk);
+    const int64_t ws = (int64_t)workspace_bytes(3 * nodes, width, prec, 2 * num_sms, pk, patterns);
     return (mesh + sys + pat + rhs + ws) * 11 / 10 + (1 << 20);
 }
 
@@ -204,7 +210,7 @@ fe_status build_request(fe_server* S, ServeReq* q) {
     if (q->mesh->n_act > 0)
         FE_CUDA(cudaMemcpyAsync(q->node_id.data(), q->mesh->node_id.ptr, q->node_id.size() * sizeof(int32_t),
                                 cudaMemcpyDeviceToHost, c->stream));
-    FE_TRY(fe_assemble(c, q->mesh, q->freq, S->so.precision, &q->sys));
+    FE_TRY(assemble_system(c, q->mesh, q->freq, S->so.precision, q->patterns, &q->sys));
     const int nrhs = (int)q->waves.size();
     DevBuf B, wave_buf;
     FE_TRY(dev_alloc(c->stream, B, (size_t)q->n_dof * nrhs * sizeof(double2)));
@@ -541,7 +547,11 @@ fe_status fe_serve_submit(fe_server* S, const fe_request* r, uint64_t* ticket) {
     }
     q->freq = r->freq_hz;
     q->width = tile_width(r->nrhs);
-    q->est_bytes = estimate_bytes(d, r->nrhs, q->width, S->o.precision, S->ictx->num_sms);
+    q->est_bytes = estimate_bytes(d, r->nrhs, q->width, S->o.precision, S->ictx->num_sms, true);
+    if (q->est_bytes > S->stats.budget_bytes) {  // (set at creation)
+        q->patterns = false;
+        q->est_bytes = estimate_bytes(d, r->nrhs, q->width, S->o.precision, S->ictx->num_sms, false);
+    }
     {
         std::lock_guard<std::mutex> lk(S->mu);
         if (S->stop) {

@@ -149,7 +149,7 @@ static size_t pat_partial_bytes(int max_cta, int R) {
 }
 
 static fe_status alloc_workspace(cudaStream_t st, int64_t n_dof, int R, int prec, int max_cta, Workspace& w,
-                                 int64_t pk_entries = 0) {
+                                 int64_t pk_entries, bool pat) {
     const size_t esz = inner_bytes(prec);  // inner-precision vectors (uM, w)
     const size_t nv = (size_t)n_dof * R;
     for (auto pr : {std::make_pair(&w.b, nv * sizeof(double2)), std::make_pair(&w.x, nv * sizeof(double2)),
@@ -159,7 +159,8 @@ static fe_status alloc_workspace(cudaStream_t st, int64_t n_dof, int R, int prec
                     std::make_pair(&w.pM, split_copies(prec, R) ? nv * esz : (size_t)16), std::make_pair(&w.w, nv * esz),
                     std::make_pair(&w.partial, (size_t)max_cta * kMaxNV * R * sizeof(double)),
                     std::make_pair(&w.result, (size_t)kMaxNV * R * sizeof(double)),
-                    std::make_pair(&w.pat, pat_partial_bytes(max_cta, R)), std::make_pair(&w.sync, sync_bytes(max_cta)),
+                    std::make_pair(&w.pat, pat ? pat_partial_bytes(max_cta, R) : (size_t)16),
+                    std::make_pair(&w.sync, sync_bytes(max_cta)),
                     std::make_pair(&w.rep, (size_t)R * (3 * sizeof(int) + sizeof(double)) + 64)}) {
         const fe_status e = dev_alloc(st, *pr.first, pr.second);
         if (e != FE_OK) {
@@ -178,12 +179,11 @@ static fe_status alloc_workspace(cudaStream_t st, int64_t n_dof, int R, int prec
 }
 
 // Bytes alloc_workspace takes (before allocator rounding).
-size_t workspace_bytes(int64_t n_dof, int R, int prec, int max_cta, int64_t pk_entries) {
+size_t workspace_bytes(int64_t n_dof, int R, int prec, int max_cta, int64_t pk_entries, bool pat) {
     const size_t nv = (size_t)n_dof * R;
     const size_t esz = inner_bytes(prec);
     return nv * (6 * sizeof(double2) + (split_copies(prec, R) ? 3 : 1) * esz) + (size_t)(max_cta + 1) * kMaxNV * R * sizeof(double) +
-           (size_t)R * 32 + 4096 + (size_t)pk_entries * esz +
-           pat_partial_bytes(max_cta, R);
+           (size_t)R * 32 + 4096 + (size_t)pk_entries * esz + (pat ? pat_partial_bytes(max_cta, R) : 0);
 }
 
 // Solve parameters for a tile of R columns held in workspace w (n_cta and the
@@ -400,7 +400,7 @@ static fe_status solve_tiles(fe_ctx* ctx, const fe_system* s, int nrhs, int ldb,
     const int prec = o.precision;
     Workspace w;
     auto cleanup = [&]() { free_workspace(st, w); };
-    fe_status e = alloc_workspace(st, n_dof, R, prec, 2 * ctx->num_sms, w, packed_entries(s, prec, R));
+    fe_status e = alloc_workspace(st, n_dof, R, prec, 2 * ctx->num_sms, w, packed_entries(s, prec, R), s->n_pat > 0);
     if (e != FE_OK) return e;
     const bool tracing = getenv("FE_TRACE") && getenv("FE_TRACE")[0] == '1';
     const size_t trace_bytes =
@@ -532,7 +532,8 @@ fe_status job_create(fe_ctx* ctx, const fe_system* s, int nrhs, const double2* d
     j->prec = prec;
     j->n_dof = 3 * (int64_t)s->mesh->n_act;
     cudaStream_t st = ctx->stream;
-    fe_status e = alloc_workspace(st, j->n_dof, j->R, prec, 2 * ctx->num_sms, j->w, packed_entries(s, prec, j->R));
+    fe_status e = alloc_workspace(st, j->n_dof, j->R, prec, 2 * ctx->num_sms, j->w, packed_entries(s, prec, j->R),
+                                  s->n_pat > 0);
     if (e != FE_OK) {
         delete j;
         return e;

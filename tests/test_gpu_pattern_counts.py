@@ -151,3 +151,25 @@ def test_tuned_choice_is_kept_per_kind_of_kernel(fe, ctx):
             fe.fe_system_destroy(s)
             fe.fe_mesh_destroy(m)
     assert how == [1, 1, 2, 2]
+
+
+# a request's device memory without patterns (8^3 elements, two waves), by precision
+@pytest.mark.parametrize("precision,budget", [("DF", 8483037), ("FP64", 5360656), ("MIXED", 6960337)])
+def test_serve_budget_without_room_for_patterns(fe, ctx, precision, budget):
+    """A budget that holds a request without its row patterns serves it, and one byte less refuses it."""
+    prob = W.pec_box_problem(8, 3e9, np.random.default_rng(8))
+    waves = W.random_waves(2, np.random.default_rng(1))
+    out = []
+    for b in (budget, budget - 1, 0):
+        srv = fe.fe_serve_create(ctx, fe.serve_opts(precision=getattr(fe, f"FE_PREC_{precision}"), hbm_budget=b))
+        try:
+            out.append(fe.fe_serve_wait(srv, fe.fe_serve_submit(srv, prob, waves), timeout_s=60.0))
+            assert fe.fe_serve_info(srv)["peak_admitted_bytes"] <= (b or 1 << 62)
+        finally:
+            fe.fe_serve_destroy(srv)
+    assert out[0]["status"] == 0, out[0]["message"]
+    assert out[1]["status"] == fe.FE_ERR_OOM and "budget" in out[1]["message"]
+    maps = fem.mesh_maps(prob)
+    A, B = fem.assemble(prob, maps=maps), fem.rhs(prob, waves, maps=maps)
+    for r in (out[0], out[2]):
+        assert fem.true_relative_residual(A, r["x"], B).max() <= 1e-8
