@@ -308,11 +308,14 @@ __device__ __noinline__ void build_pat_tables(const SolveParams& P, int pr0, int
                                 info_word(t, loc[pid], ord[pid]));
         }
         __syncthreads();
-        // four rows in a row of the grid with one pattern
-        for (int i = halo->first_diag + 4 * tid; i + 3 < n; i += 4 * kPT)
-            if (info[i + 3].y - info[i].y == 3 && info[i + 1].z == info[i].z && info[i + 2].z == info[i].z &&
-                info[i + 3].z == info[i].z)
-                info[i].w |= kInfoQuad;
+        // four rows in a row of the grid with one pattern: equal places and equal
+        // words (a place is in the shared copy or in the global list, as bit
+        // kInfoShared says); a row's own word is changed by its four's thread only
+        for (int i = halo->first_diag + 4 * tid; i + 3 < n; i += 4 * kPT) {
+            bool same = info[i + 3].y - info[i].y == 3;
+            for (int k = 1; k < 4; ++k) same = same && info[i + k].z == info[i].z && info[i + k].w == info[i].w;
+            if (same) info[i].w |= kInfoQuad;
+        }
         // lines of the rows; a line outside the box or with an inactive centre
         // node carries no term and points at the row itself
         const int ny1 = P.pat_sz / P.pat_sy;
