@@ -198,11 +198,11 @@ __global__ void k_face_flags(const uint8_t* __restrict__ mat, Grid g, unsigned a
     fpec[t] = ispec;
 }
 
-__global__ void k_face_compact(const int* __restrict__ flag, const int* __restrict__ pos, int* __restrict__ out,
-                               int64_t n) {
+// pos: scanned in place over the flags, so that a face is listed where the
+// next position (the total behind the last) is another.
+__global__ void k_face_compact(const int* __restrict__ pos, int total, int* __restrict__ out, int64_t n) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n) return;
-    if (flag[t]) out[pos[t]] = (int)t;
+    if (t < n && (t + 1 < n ? pos[t + 1] : total) != pos[t]) out[pos[t]] = (int)t;
 }
 
 static unsigned blocks_for(int64_t n, int threads) { return (unsigned)((n + threads - 1) / threads); }
@@ -267,32 +267,31 @@ static fe_status build(fe_ctx* ctx, fe_mesh* m) {
     FE_TRY(scan_exclusive(st, rp, rp, m->n_act, d_small + 2, ctx->scan_tmp));
     FE_CUDA(cudaMemcpyAsync(rp + m->n_act, d_small + 2, sizeof(int), cudaMemcpyDeviceToDevice, st));
 
-    // Faces: both lists are counted before the one synchronisation that sizes
-    // them and the column indices.
+    // Faces: both lists are counted, in place of their flags, before the one
+    // synchronisation that sizes them and the column indices.
     int* fext = fl;
-    DevBuf fpec_flags, pos, pos_pec;
+    DevBuf fpec_flags;
     FE_TRY(dev_alloc(st, fpec_flags, (size_t)(6 * ne) * sizeof(int)));
-    FE_TRY(dev_alloc(st, pos, (size_t)(6 * ne) * sizeof(int)));
-    FE_TRY(dev_alloc(st, pos_pec, (size_t)(6 * ne) * sizeof(int)));
+    int* fpec = (int*)fpec_flags.ptr;
     k_face_flags<<<blocks_for(6 * ne, 256), 256, 0, st>>>((const uint8_t*)m->material.ptr, g,
-                                                          abc_faces(m->boundary), fext, (int*)fpec_flags.ptr, ne);
+                                                          abc_faces(m->boundary), fext, fpec, ne);
     FE_LAUNCHED();
-    FE_TRY(scan_exclusive(st, fext, (int*)pos.ptr, 6 * ne, d_small + 3, ctx->scan_tmp));
-    FE_TRY(scan_exclusive(st, (const int*)fpec_flags.ptr, (int*)pos_pec.ptr, 6 * ne, d_small + 4, ctx->scan_tmp));
+    FE_TRY(scan_exclusive(st, fext, fext, 6 * ne, d_small + 3, ctx->scan_tmp));
+    FE_TRY(scan_exclusive(st, fpec, fpec, 6 * ne, d_small + 4, ctx->scan_tmp));
     FE_CUDA(cudaMemcpyAsync(h_small + 2, d_small + 2, 3 * sizeof(int), cudaMemcpyDeviceToHost, st));
     FE_CUDA(cudaStreamSynchronize(st));
     m->nnzb = h_small[2];
     m->n_ext = h_small[3];
     m->n_pec = h_small[4];
     FE_TRY(dev_alloc(st, m->faces_ext, (size_t)m->n_ext * sizeof(int)));
-    k_face_compact<<<blocks_for(6 * ne, 256), 256, 0, st>>>(fext, (const int*)pos.ptr, (int*)m->faces_ext.ptr,
-                                                            6 * ne);
+    k_face_compact<<<blocks_for(6 * ne, 256), 256, 0, st>>>(fext, (int)m->n_ext, (int*)m->faces_ext.ptr, 6 * ne);
     FE_LAUNCHED();
     FE_TRY(dev_alloc(st, m->faces_pec, (size_t)m->n_pec * sizeof(int)));
-    k_face_compact<<<blocks_for(6 * ne, 256), 256, 0, st>>>((const int*)fpec_flags.ptr, (const int*)pos_pec.ptr,
-                                                            (int*)m->faces_pec.ptr, 6 * ne);
+    k_face_compact<<<blocks_for(6 * ne, 256), 256, 0, st>>>(fpec, (int)m->n_pec, (int*)m->faces_pec.ptr, 6 * ne);
     FE_LAUNCHED();
 
+    dev_free(st, flags);
+    dev_free(st, fpec_flags);
     FE_TRY(dev_alloc(st, m->col_idx, (size_t)m->nnzb * sizeof(int)));
     k_col_fill<<<blocks_for(((int64_t)m->n_act + 3) / 4 * 32, 256), 256, 0, st>>>(
         g, (const int*)m->node_id.ptr, (const int*)m->node_rank.ptr, (const unsigned*)mask.ptr, rp,
@@ -303,10 +302,6 @@ static fe_status build(fe_ctx* ctx, fe_mesh* m) {
                                                          (const int*)m->node_rank.ptr, (const unsigned*)mask.ptr, rp,
                                                          (int*)m->elem_slot.ptr, ne);
     FE_LAUNCHED();
-    dev_free(st, flags);
-    dev_free(st, fpec_flags);
-    dev_free(st, pos);
-    dev_free(st, pos_pec);
     dev_free(st, mask);
     m->bytes = (int64_t)(m->material.bytes + m->node_rank.bytes + m->node_id.bytes + m->row_ptr.bytes +
                          m->col_idx.bytes + m->elem_slot.bytes + m->faces_ext.bytes + m->faces_pec.bytes);
