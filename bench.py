@@ -229,13 +229,25 @@ def product_bytes(info, s, R):
 # x 2.07 GHz; FP64 issues at 1/64 of the FP32 rate on GB300.
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12   # 80.5 (an FMA loop on the box measured 72)
 FP64_PEAK_TFLOPS = FP32_PEAK_TFLOPS / 64            # 1.26 (measured 1.20)
+# instructions of one row-pattern term (a real weight times a complex entry): two FMA, or in FP32 pairs two
+# multiplications with their errors and two pair additions
+TERM_INSTRUCTIONS = {"fp64": 2, "mixed": 2, "df": 24}
+
+
+def executed_share(base, terms, columns, products, launch_s):
+    """Instructions a second of the products that a launch on row patterns executes (in 10^12), their pipe's rate, and
+    the share of it: the vector updates and inner products come on top."""
+    peak = (FP64_PEAK_TFLOPS if base == "fp64" else FP32_PEAK_TFLOPS) / 2.0
+    rate = products * terms * columns * TERM_INSTRUCTIONS[base] / launch_s / 1e12 if launch_s > 0 else None
+    return rate, peak, rate / peak if rate is not None else None
 
 
 def kernel_hash() -> str:
     import hashlib
     csrc = ROOT / "paper_0704_2344_gb300" / "csrc"
     h = hashlib.sha256()
-    for f in ("solve.cu", "solve_kernels.cuh", "solve_pattern.cuh", "patterns.cuh", "krylov.cuh", "fe_internal.cuh"):
+    for f in ("solve.cu", "solve_kernels.cuh", "solve_pattern.cuh", "patterns.cuh", "row_cost.cuh", "krylov.cuh",
+              "fe_internal.cuh"):
         h.update((csrc / f).read_bytes())
     return h.hexdigest()[:16]
 
@@ -321,6 +333,7 @@ def run_ours(args, rank, world, local_rank, precision_name):
     info = fe.fe_mesh_info(mesh0)
     sys0 = fe.fe_assemble(ctx, mesh0, prob.freq_hz, precision)
     sysinfo = fe.fe_system_info(sys0)
+    n_patterns, terms = fe.fe_system_patterns(ctx, sys0)
     bicp_blocks, bicp_factor_ms = 0, None
     if bicp:  # strictly lower blocks inside the bands: the substitutions' work
         t_f = time.perf_counter()
@@ -394,9 +407,6 @@ def run_ours(args, rank, world, local_rank, precision_name):
               "product_flops_per_launch": int(fl_prod / args.steps), "fp64_flops_per_launch": int(fl64 / args.steps),
               "product_rows": dict(zip(("blocks_explicit", "rows_general", "rows_diagonal"),
                                        product_rows(sysinfo, base)))}
-    if bicp:
-        common["bicp_band_blocks"] = bicp_blocks
-        common["bicp_factor_ms"] = round(bicp_factor_ms, 3)
     # The roofline of the method's own work (every stored block, the row
     # pointers and the input and output vectors once per product; 8 flops per
     # complex multiply-add), not of the arithmetic that implements it.
@@ -411,33 +421,56 @@ def run_ours(args, rank, world, local_rank, precision_name):
             "method_bytes_per_launch": int(method_bytes), "method_flops_per_launch": int(method_flops),
             "entry_bytes": s_inner, "columns_per_launch": tile_w}
     launch_s = launch_ms * 1e-3
-    if base == "fp64":
-        # complex128 products run on the FP64 pipes (1/64 of the FP32 rate):
-        # 8 flops per complex multiply-add against that rate
-        achieved = method_flops / launch_s / 1e12 if launch_s > 0 else None
-        roof = {"kernel": f"{'k_solve' if bicp else 'k_solve_pat'}<double,{tile_w}> (persistent COCG, FP64"
-                          + (", block incomplete Cholesky)" if bicp else ")"), "bound": "alu",
-                "achieved": round(achieved, 4) if achieved else None, "peak": round(FP64_PEAK_TFLOPS, 3),
-                "unit": "TFLOP/s", "frac": round(achieved / FP64_PEAK_TFLOPS, 4) if achieved else None,
-                "peak_source": "FP64 rate from unit counts and clock (an FMA loop measured 1.20)",
-                "work": "method_flops_per_launch / (launch_ms * 1e-3) / 1e12",
-                "hbm_view": {"achieved_gbs": round(method_bytes / launch_s / 1e9, 1), "peak_gbs": hbm_peak,
-                             "frac": round(method_bytes / launch_s / 1e9 / hbm_peak, 4)} if launch_s > 0 else None}
+    method_view = {"gbs": round(method_bytes / launch_s / 1e9, 1), "hbm_peak_gbs": hbm_peak,
+                   "hbm_frac": round(method_bytes / launch_s / 1e9 / hbm_peak, 4),
+                   "tflops": round(method_flops / launch_s / 1e12, 3),
+                   "fp64_peak_tflops" if base == "fp64" else "fp32_peak_tflops":
+                       round(FP64_PEAK_TFLOPS if base == "fp64" else FP32_PEAK_TFLOPS, 3),
+                   "peak_source": f"{hbm_src} (MEASURED_PEAKS.json hbm_gbs)" if hbm_src == "measured" else hbm_src,
+                   } if launch_s > 0 else None
+    if n_patterns and not bicp:
+        # What the launch executes: products read the non-zero terms of the row
+        # patterns, in shared memory, not the stored blocks.  The method's own
+        # work per second (every block read, every multiply-add done) can
+        # therefore exceed the hardware's rates and stands beside it.
+        rate, peak, frac = executed_share(base, terms, tile_w, prod_inner / steps, launch_s)
+        roof = {"kernel": f"k_solve_pat<{ {'fp64': 'double', 'df': 'DFloat', 'mixed': 'float'}[base]},{tile_w}> "
+                          "(persistent COCG on row patterns)", "bound": "latency",
+                "achieved": round(rate, 4) if rate else None, "peak": round(peak, 4), "unit": "T instructions/s",
+                "frac": round(frac, 4) if frac else None,
+                "peak_source": ("FP64" if base == "fp64" else "FP32") + " pipe from unit counts and clock",
+                "work": "products_per_launch * terms_per_product * columns_per_launch * instructions_per_term / "
+                        "(launch_ms * 1e-3) / 1e12",
+                "patterns": n_patterns, "terms_per_product": terms, "instructions_per_term": TERM_INSTRUCTIONS[base],
+                "method_view": method_view}
+        roof.update(work)
     else:
-        achieved = method_bytes / launch_s / 1e9 if launch_s > 0 else None
-        roof = {"kernel": f"k_solve_pat<{'DFloat' if base == 'df' else 'float'},{tile_w}> (persistent COCG, "
-                          + ("FP32-pair" if base == "df" else "complex64") + " products)", "bound": "hbm",
-                "achieved": round(achieved, 1) if achieved else None, "peak": hbm_peak, "unit": "GB/s",
-                "frac": round(achieved / hbm_peak, 4) if achieved else None,
-                "peak_source": f"{hbm_src} (MEASURED_PEAKS.json hbm_gbs)" if hbm_src == "measured" else hbm_src,
-                "work": "(products_per_launch * bytes_per_product + fp64_products_per_launch * "
-                        "bytes_per_fp64_product) / (launch_ms * 1e-3) / 1e9",
-                "note": "the method's bytes; products from row patterns do not read the stored blocks",
-                "alu_view": {"method_tflops": round(method_flops / launch_s / 1e12, 3) if launch_s > 0 else None,
-                             "fp32_peak_tflops": round(FP32_PEAK_TFLOPS, 2)}}
-    roof.update(work)
-    roof["stencil_reduced_bytes_per_launch"] = int(alg / steps)   # what products from per-material stencils read
-    roof.update(common)
+        if base == "fp64":
+            # complex128 products run on the FP64 pipes (1/64 of the FP32 rate):
+            # 8 flops per complex multiply-add against that rate
+            achieved = method_flops / launch_s / 1e12 if launch_s > 0 else None
+            roof = {"kernel": f"k_solve<double,{tile_w}> (persistent COCG, FP64"
+                              + (", block incomplete Cholesky)" if bicp else ")"), "bound": "alu",
+                    "achieved": round(achieved, 4) if achieved else None, "peak": round(FP64_PEAK_TFLOPS, 3),
+                    "unit": "TFLOP/s", "frac": round(achieved / FP64_PEAK_TFLOPS, 4) if achieved else None,
+                    "peak_source": "FP64 rate from unit counts and clock (an FMA loop measured 1.20)",
+                    "work": "method_flops_per_launch / (launch_ms * 1e-3) / 1e12"}
+        else:
+            achieved = method_bytes / launch_s / 1e9 if launch_s > 0 else None
+            roof = {"kernel": f"k_solve<{'DFloat' if base == 'df' else 'float'},{tile_w}> (persistent COCG, "
+                              + ("FP32-pair" if base == "df" else "complex64") + " products)", "bound": "hbm",
+                    "achieved": round(achieved, 1) if achieved else None, "peak": hbm_peak, "unit": "GB/s",
+                    "frac": round(achieved / hbm_peak, 4) if achieved else None,
+                    "peak_source": f"{hbm_src} (MEASURED_PEAKS.json hbm_gbs)" if hbm_src == "measured" else hbm_src,
+                    "work": "(products_per_launch * bytes_per_product + fp64_products_per_launch * "
+                            "bytes_per_fp64_product) / (launch_ms * 1e-3) / 1e9"}
+        roof["method_view"] = method_view
+        roof.update(work)
+        roof["stencil_reduced_bytes_per_launch"] = int(alg / steps)   # what products from per-material stencils read
+        roof.update(common)
+    if bicp:
+        roof["bicp_band_blocks"] = bicp_blocks
+        roof["bicp_factor_ms"] = round(bicp_factor_ms, 3)
     roof["traffic"] = recorded_traffic(args.workload, precision_name)   # ncu DRAM bytes per launch (or None)
     roof["launch_ms"] = round(launch_ms, 4)
     roof["kernel_share_of_step"] = round(kernel_ms / total_ms, 4) if total_ms else None
@@ -569,8 +602,10 @@ def run_spmv(args, rank, world, local_rank):
         "scaling": "weak", "vs_baseline": None, "dtype": "c64", "data": "synthetic",
         "config": {"workload": f"{args.workload}: {prob.name}, {n_dof} unknowns, {nnzb} blocks",
                    "l2": "512 MiB flush before every timed product", "parallelism": f"replicas x{world}"},
-        "roofline": {"kernel": "k_spmv_warp<float2> (warp per block row, lane per block)", "bound": "hbm",
+        "roofline": {"kernel": "fe_spmv, complex64, one column (row patterns; the form by the size)", "bound": "l1",
                      "achieved": head["gbs"], "peak": hbm_peak, "unit": "GB/s", "frac": head["frac_hbm"],
+                     "note": "bytes of the stored blocks, which products on row patterns do not read: the fraction can "
+                             "exceed one; fe_spmv_half reads its blocks",
                      "traffic": None, "algorithmic_bytes_per_launch": head["bytes"]},
         "table": table, "gpu_launches": fe.fe_launch_count() - launches0, "timed_launches": n_timed,
         "e2e": None, "clocks": clk.summary(),
