@@ -407,9 +407,10 @@ __global__ void __launch_bounds__(256) k_spmv_pat(PatView<C> V, int n_rows, cons
 
 // split: K lanes per item, K R columns (a power of two up to 32) per warp part.
 // The row's own entry, the last step of its lane, goes last of all: that lane
-// adds it to the sum of all lanes and stores the result.  In grid order the error of random vectors was up to
-// 1.4 times that of the stored blocks (31^3 elements, one column, FP32 pairs
-// 5.6e-15, 4.0e-15 now, 4.2e-15 by blocks); 9 261 rows 4.75 us so, 4.1 now.
+// adds it to the sum of all lanes and stores the result.  In grid order the
+// error of random vectors was up to 1.4 times that of the stored blocks (31^3
+// elements, one column, FP32 pairs 5.6e-15, 4.0e-15 now, 4.2e-15 by blocks);
+// 9 261 rows 4.75 us so, 4.1 now.
 template <typename C, int R, int K>
 __global__ void __launch_bounds__(256) k_spmv_pat_split(PatView<C> V, int n_rows, const C* __restrict__ x,
                                                         C* __restrict__ y) {
@@ -564,30 +565,30 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_spmv_pat_tile(PatView<float
 // Form of a product of `rows` rows and R columns on `lanes` resident lanes
 // (2 048 per SM, 311 296), by its items n = 3 rows R.  Lanes share an item while
 // that does not take more than the chip's: 8 up to n = lanes / 8, 4 up to
-// lanes / 4, 2 up to lanes / 2.  FP64 and FP32 pairs are plain above, and so is
-// complex64 of 8 columns and more until the tiles pay at n = 8 lanes; with up
-// to 4 columns complex64 keeps its weights.  Times in us per product in a
-// stream of them, on either side of a bound (cubes with a slab and a PEC body):
-//   keep    1 column 50 528 rows 12.4 shared and 14.4, 59 194 rows 14.5 and 14.4;
-//           2 columns 24 362 rows 12.3 and 14.4, 29 727 rows 14.4 and 14.4;
-//           4 columns 12 159 rows 12.3 and 14.4, 13 816 rows 14.4 and 14.4
-//   tile    8 columns 90 909 rows 50.3 plain and 49.3, 148 534 rows 75.9 and 67.8;
-//           16: 46 592 rows 53.2 and 55.1, 54 747 rows 59.5 and 55.8;
-//           32: 21 925 rows 52.1 and 50.1, 29 727 rows 65.7 and 63.5
-//           and 8 columns up to n = 2 lanes: 15 598 rows 20.5 and 18.5, 24 362 rows
-//           22.4 and 20.6, 26 973 rows 22.6 and 26.2
+// lanes / 4, 2 up to lanes / 2.  FP64 and FP32 pairs are plain above; complex64 is
+// plain until the walks pay: from n = lanes with up to 4 columns, from 3.5
+// lanes with 8 and 32, from 5 lanes with 16.  A walk takes every SM whole, so that
+// products on several streams do not overlap; both ways count.  Times in us
+// per product, of systems on three streams in turn / of one alone, on either
+// side of a bound (cubes with a slab and a PEC body):
+//   1 column    90 909 rows  plain 8.2 / 19, walk 10.6 / 19; 117 306  8.1 / 19, 11.3 / 16
+//   2 columns   50 528 rows  plain 8.3 / 21, walk 10.7 / 14; 68 796   9.3 / 21, 11.9 / 16
+//   4 columns   24 362 rows  plain 8.2 / 19, walk 10.6 / 14; 35 873  10.2 / 21, 12.0 / 16
+//   8 columns   42 811 rows  plain 22.9 / 29, walk 24.4 / 31; 68 796  36.1 / 40, 33.7 / 44
+//   16 columns  29 727 rows  plain 31.6 / 37, walk 30.6 / 39; 35 873  39.2 / 43, 35.4 / 43
+//   32 columns  10 640 rows  plain 24.2 / 29, walk 24.5 / 37; 15 598  36.2 / 41, 32.5 / 41
 // The stored blocks of a small system stay in L2, and a warp reads a row's
 // blocks at once, so that their chain of dependent loads is one shorter than a
 // pattern's (row, line, term, entry).  They round more (complex64 of 8 columns
 // and more 1.0e-7 against 4.6e-8), so they are taken only where the patterns
-// are clearly slower:
+// are clearly slower, all systems alone:
 //   complex64  1 column n <= lanes / 9: 10 640 rows 6.5 stored and 8.2, 12 159 8.2 and 8.2
 //              2 columns n <= lanes / 5: 9 253 rows 8.2 and 8.3, 10 640 8.3 and 8.3
 //              8 and 16 columns from lanes / 2 to 4/5 lanes, between the shared
 //              items and the others: 8 columns 9 253 rows 12.4 and 16.4; 16 columns
 //              4 912 rows 14.4 and 18.5
-//   FP32 pairs 1 and 4 columns n <= lanes / 32: 2 196 rows 6.2 and 8.0, 3 374 8.2 and
-//              7.3; 4 columns 512 rows 6.3 and 6.7, 1 331 8.2 and 8.2
+//   FP32 pairs 1 and 4 columns n <= lanes / 40: 2 196 rows 6.2 and 7.3, 2 743 7.7 and
+//              7.4; 4 columns 512 rows 6.3 and 7.2, 1 000 rows 7.3 and 7.3
 enum class Form { kStored, kSplit8, kSplit4, kSplit2, kPlain, kWalk };
 
 static Form product_form(int precision, int64_t rows, int R, int sms) {
@@ -597,11 +598,12 @@ static Form product_form(int precision, int64_t rows, int R, int sms) {
     if (c64 && ((R == 1 && 9 * n <= lanes) || (R == 2 && 5 * n <= lanes) ||
                 ((R == 8 || R == 16) && 2 * n > lanes && 5 * n <= 4 * lanes)))
         return Form::kStored;
-    if (precision == FE_PREC_DF && (R == 1 || R == 4) && 32 * n <= lanes) return Form::kStored;
+    if (precision == FE_PREC_DF && (R == 1 || R == 4) && 40 * n <= lanes) return Form::kStored;
     if (8 * R <= 32 && 8 * n <= lanes) return Form::kSplit8;
     if (4 * R <= 32 && 4 * n <= lanes) return Form::kSplit4;
     if (2 * R <= 32 && 2 * n <= lanes) return Form::kSplit2;
-    return c64 && (R <= 4 || (R == 8 && n <= 2 * lanes) || n > 8 * lanes) ? Form::kWalk : Form::kPlain;
+    const double walk_from = R <= 4 ? lanes : (R == 16 ? 5.0 : 3.5) * lanes;
+    return c64 && n > walk_from ? Form::kWalk : Form::kPlain;
 }
 
 template <typename C, int R>
