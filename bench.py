@@ -582,6 +582,11 @@ def run_spmv(args, rank, world, local_rank):
                     table[f"{pname}_R{R}"] = {"ms": round(ms, 4), "gbs": round(by / ms / 1e6, 1),
                                              "frac_hbm": round(by / ms / 1e6 / hbm_peak, 4),
                                              "tflops": round(fl / ms / 1e9, 3), "bytes": int(by)}
+                    if fe.fe_system_patterns(ctx, system)[0]:
+                        # what a product on row patterns has to move: the vectors and 22 bytes of tables a row
+                        moved = 2 * n_dof * R * esz + 22 * n
+                        table[f"{pname}_R{R}"] |= {"moved_bytes": int(moved),
+                                                   "moved_frac_hbm": round(moved / ms / 1e6 / hbm_peak, 4)}
                     if kept:
                         # half storage: kept blocks, every column index, the transposed
                         # slot of each upper block, row pointers of both layouts, vectors

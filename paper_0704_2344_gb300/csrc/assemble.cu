@@ -8,8 +8,9 @@
 // (k_tables), plus per face orientation the absorbing-boundary form G of
 // Eq. 3 and the penalty surface term of Eq. 4.  The assembly kernel then
 // follows the paper's assembly by degree of freedom (Section 3.1.2): one warp
-// per node (with row patterns: per distinct row, the others being copies) gathers, for each of the node's up to 27 blocks, the contributions
-// of the elements and faces shared with the neighbour, with no atomics.  The
+// per node (with row patterns: per distinct row, the others being copies)
+// gathers, for each of the node's up to 27 blocks, the contributions of the
+// elements and faces shared with the neighbour, with no atomics.  The
 // symmetrisation by the transpose (Section 3.1.4, variant P) is applied to
 // each face table, since (sum_e A_e)^T = sum_e A_e^T.  The same warp inverts
 // the diagonal block for the block-Jacobi preconditioner.

@@ -15,7 +15,7 @@
 // read the stored blocks.  Bound by launches and dependent loads, but for the
 // copies (k_pat_spread: two stored forms of 51^3 rows, 1 GB).  Mesh, assembly,
 // four right-hand sides and a product of 51^3 nodes: 7.5 ms with every row
-// assembled, 1.6 ms with the first rows only, 0.76 ms with the right-hand side
+// assembled, 1.6 ms with the first rows only, 0.75 ms with the right-hand side
 // and the other set-up kernels shortened.
 #include "patterns.cuh"
 
@@ -355,8 +355,8 @@ fe_status group_rows(fe_ctx* ctx, fe_system* s, DevBuf& row_group, int* d_flags)
     const unsigned grid = (unsigned)((n + 255) / 256);
     const int limit = pat_limit(m->n_nodes_total);
     k_pat_insert<<<grid, 256, 0, st>>>((const uint8_t*)m->material.ptr, m->nx, m->ny, m->nz,
-                                       (const int*)m->node_id.ptr, n, far, limit, (RowKey*)row_keys.ptr, (unsigned long long*)keys.ptr, (int*)first.ptr,
-                                       (int*)slot_of.ptr, d_flags);
+                                       (const int*)m->node_id.ptr, n, far, limit, (RowKey*)row_keys.ptr,
+                                       (unsigned long long*)keys.ptr, (int*)first.ptr, (int*)slot_of.ptr, d_flags);
     k_pat_number<<<1, 1024, 0, st>>>((const unsigned long long*)keys.ptr, (const int*)first.ptr, limit,
                                      (int*)id_of_slot.ptr, (int*)s->pat_first.ptr, d_flags);
     k_pat_group<<<grid, 256, 0, st>>>((const RowKey*)row_keys.ptr, (const int*)slot_of.ptr,

@@ -16,12 +16,13 @@
 //     mid-sized system has some 600 items, so the phases are bound by latency,
 //     and registers for loads in flight count more than warps.
 //
-// Bound by latency: of the 16.5 us an iteration of the 3-wavelength cube takes
-// with FP32 pairs, the two grid barriers take 4.3 and the rest is short phases
-// of dependent operations; FP64 keeps its pipe about half busy.  Measured, us
-// per iteration, solve_kernels.cuh and here: FP32 pairs 10^3 20.1 and 10.7, 30^3
-// 25.6 and 16.5, 40^3 expanded 90 and 26.7, 18^3 with 12 columns 106 and 36;
-// FP64 20^3 48 and 19.6; complex64 20^3 14.6 (17.4 before its sums were paired).
+// Bound by latency: of the 16.2 us an iteration of the 3-wavelength cube takes
+// with FP32 pairs, the reduction with its barrier takes 3.8 and the second
+// barrier 1.95, and the rest is short phases of dependent operations; FP64 keeps
+// its pipe about half busy.  Measured, us per iteration, solve_kernels.cuh and
+// here: FP32 pairs 10^3 20.1 and 10.7, 30^3 25.6 and 16.2, 40^3 expanded 90 and
+// 26.7, 18^3 with 12 columns 106 and 36; FP64 20^3 48 and 19.6; complex64 20^3
+// 14.6 (16.7 before its sums were paired).
 #pragma once
 
 #include "solve_kernels.cuh"
@@ -74,7 +75,7 @@ __device__ __forceinline__ bool pat_barrier(const SolveParams& P, unsigned& pass
 // the barrier's parity: a CTA writes those of barrier e + 2 only after every
 // CTA has arrived at barrier e + 1, that is after it has read barrier e's.
 // (Words that carry their own number, polled by every CTA instead of a
-// counter, were slower: 4.5 us against 2.9 us on 152 CTAs, the polls of all
+// counter, were slower: 4.5 us against 2.2 to 2.5 us on 152 CTAs, the polls of all
 // CTAs on the same few lines delaying the stores they wait for.)
 template <int NV, bool kPair>
 __device__ __noinline__ bool pat_reduce(const SolveParams& P, int cta, const double* s_in, double* s_out,
