@@ -410,7 +410,9 @@ __global__ void __launch_bounds__(256) k_spmv_pat(PatView<C> V, int n_rows, cons
 // adds it to the sum of all lanes and stores the result.  In grid order the
 // error of random vectors was up to 1.4 times that of the stored blocks (31^3
 // elements, one column, FP32 pairs 5.6e-15, 4.0e-15 now, 4.2e-15 by blocks);
-// 9 261 rows 4.75 us so, 4.1 now.
+// 9 261 rows take 4.75 us so and 4.1 now; with two lanes an item the step aside
+// costs 5 to 7 % (FP32 pairs, two columns of 24^3 elements on three streams 7.3
+// and 7.7 us).
 template <typename C, int R, int K>
 __global__ void __launch_bounds__(256) k_spmv_pat_split(PatView<C> V, int n_rows, const C* __restrict__ x,
                                                         C* __restrict__ y) {
@@ -565,8 +567,9 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_spmv_pat_tile(PatView<float
 // Form of a product of `rows` rows and R columns on `lanes` resident lanes
 // (2 048 per SM, 311 296), by its items n = 3 rows R.  Lanes share an item while
 // that does not take more than the chip's: 8 up to n = lanes / 8, 4 up to
-// lanes / 4, 2 up to lanes / 2.  FP64 and FP32 pairs are plain above; complex64 is
-// plain until the walks pay: from n = lanes with up to 4 columns, from 3.5
+// lanes / 4, 2 up to 0.48 lanes (FP32 pairs of 50 528 rows, just beyond: 11.5 us
+// shared and 8.6 plain on three streams; 42 811 rows alone 17 and 19).  FP64 and
+// FP32 pairs are plain above; complex64 is plain until the walks pay: from n = lanes with up to 4 columns, from 3.5
 // lanes with 8 and 32, from 5 lanes with 16.  A walk takes every SM whole, so that
 // products on several streams do not overlap; both ways count.  Times in us
 // per product, of systems on three streams in turn / of one alone, on either
@@ -584,7 +587,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_spmv_pat_tile(PatView<float
 // are clearly slower, all systems alone:
 //   complex64  1 column n <= lanes / 9: 10 640 rows 6.5 stored and 8.2, 12 159 8.2 and 8.2
 //              2 columns n <= lanes / 5: 9 253 rows 8.2 and 8.3, 10 640 8.3 and 8.3
-//              8 and 16 columns from lanes / 2 to 4/5 lanes, between the shared
+//              8 and 16 columns from 0.48 to 0.8 lanes, between the shared
 //              items and the others: 8 columns 9 253 rows 12.4 and 16.4; 16 columns
 //              4 912 rows 14.4 and 18.5
 //   FP32 pairs 1 and 4 columns n <= lanes / 40: 2 196 rows 6.2 and 7.3, 2 743 7.7 and
@@ -596,12 +599,12 @@ static Form product_form(int precision, int64_t rows, int R, int sms) {
     if (R > 32 || (R & (R - 1))) return Form::kPlain;
     const bool c64 = precision == FE_PREC_MIXED;
     if (c64 && ((R == 1 && 9 * n <= lanes) || (R == 2 && 5 * n <= lanes) ||
-                ((R == 8 || R == 16) && 2 * n > lanes && 5 * n <= 4 * lanes)))
+                ((R == 8 || R == 16) && n > 0.48 * lanes && 5 * n <= 4 * lanes)))
         return Form::kStored;
     if (precision == FE_PREC_DF && (R == 1 || R == 4) && 40 * n <= lanes) return Form::kStored;
     if (8 * R <= 32 && 8 * n <= lanes) return Form::kSplit8;
     if (4 * R <= 32 && 4 * n <= lanes) return Form::kSplit4;
-    if (2 * R <= 32 && 2 * n <= lanes) return Form::kSplit2;
+    if (2 * R <= 32 && n <= 0.48 * lanes) return Form::kSplit2;
     const double walk_from = R <= 4 ? lanes : (R == 16 ? 5.0 : 3.5) * lanes;
     return c64 && n > walk_from ? Form::kWalk : Form::kPlain;
 }
